@@ -18,14 +18,14 @@
 //   P1 marker bit sets; a tile with no marker in its region only copies its
 //      colour words (P7)
 //   P2 moved point of every marker (the only global reads of fractions and
-//      velocities); corner flips (Fig. 5) by XOR into the new colour bits;
-//      every aligned edge a marker lands on is claimed once
-//   P3 landings on the claimed edges (Sec. 2.4), new aligned markers; list of
-//      the interface cells whose chords can cross the tile's grid lines
+//      velocities), kept by the marker's rank in its bit set; corner flips
+//      (Fig. 5) by XOR into the new colour bits; landing edges claimed
+//   P3 landings (Sec. 2.4), new aligned markers; list of the interface cells
+//      whose chords can cross the tile's grid lines
 //   P4 each chord of such a cell that crosses a grid line k of the tile
 //      becomes a candidate of unaligned edge (k, j): references to A, B and
 //      points 1-4, centre-rule verdicts; candidates are linked per edge
-//   P5 circle fits (Sec. 2.2) of all candidates, one per thread, so the FP64
+//   P5 circle fits (Sec. 2.2) of all candidates, two lanes each, so the FP64
 //      pipe sees full warps
 //   P6 one marker per edge from its linked candidates; new unaligned markers
 //   P7 centre colours of the new four-marker cells (Sec. 2.3); colour words
@@ -48,13 +48,24 @@ template <int CAP> __host__ __device__ constexpr uint32_t head_none() {
   return (1u << head_bits<CAP>()) - 1u;
 }
 constexpr uint16_t kKindV = 0x8000;    // marker reference: region index | kKindV if unaligned
+constexpr int kSecond = 0x4000;        // segment reference: region index of its cell | kSecond for the
+                                       // second one of a four-marker cell
+static_assert(kRN <= kSecond, "region indices leave the flag bits free");
 
-// Block shape: 7 warps per tile; tiles resident per SM as shared memory
-// allows (4 in the FP32 form, 3 in the FP64 form).
-template <typename R> __host__ __device__ constexpr int tile_threads() { return 224; }
+// Block shape: four warps per tile, seven tiles per SM in the FP32 form (72
+// registers) and six in the FP64 form (80).  What a tile waits for is latency
+// (barriers, the state's loads, the fits' FP64 chains), so many small blocks
+// that are in different phases beat few large ones: 4096^2 cells, cellular
+// flow over 20000 disks, microseconds a sweep in FP32 / FP64 form: 257 / 301
+// with four warps, 265 / 310 with five at six and five tiles per SM, 267 / 308
+// at six and five tiles of four warps, 262 / 300 at eight and seven (spills);
+// seven warps at four and three tiles per SM, which the dense per-edge arrays
+// of moved fractions allowed before markers were kept by rank: 306 / 397.
+template <typename R> __host__ __device__ constexpr int tile_threads() { return 128; }
 template <typename R> __host__ __device__ constexpr int tile_min_blocks();
-template <> __host__ __device__ constexpr int tile_min_blocks<float>() { return 4; }
-template <> __host__ __device__ constexpr int tile_min_blocks<double>() { return 3; }
+template <> __host__ __device__ constexpr int tile_min_blocks<float>() { return 7; }
+template <> __host__ __device__ constexpr int tile_min_blocks<double>() { return 6; }
+constexpr int kMkCap = 1536;  // markers of a region held in shared memory
 // Candidates per tile of the batched kernels: many small grids of uneven
 // sizes hold more interface per tile than one large grid, and the longer
 // list (16-bit heads) still leaves 4 (FP32) / 3 (FP64) tiles per SM.
@@ -71,7 +82,6 @@ template <typename R> __host__ __device__ constexpr int batch_cand_cap() {
 enum { CF_P1 = 1, CF_P4 = 4, CF_OWNED = 16 };
 struct Cand {
   double y;
-  float sf;  // the crossing as an FP32 marker fraction (FP32 state only)
   uint16_t a, b, p1, p4;
   uint16_t edge;  // (j - j0) * (kTI + 1) + (k - i0)
   uint8_t fl, ord;
@@ -79,52 +89,52 @@ struct Cand {
 };
 
 // Shared memory of one tile (dynamic).  Arrays whose phases do not overlap
-// share storage: the marker lists of P1-P3 with the candidates of P4-P6, the
-// aligned / unaligned marker bit sets of P1-P3 with the candidate bit sets of
-// P4-P6, and the interface-cell list of P3-P4 with the verdicts of P6-P7.
+// share storage: the marker list of P1-P3 with the candidates of P4-P6 and the
+// interface-cell list of P3-P4 with the verdicts of P6-P7.
 template <typename R, int CAP = kCandCap>
 struct TileMem {
   static_assert(CAP <= 65534, "candidate slots fit the 16-bit heads");
   static constexpr int kCap = CAP;
   union {
-    struct {
-      uint16_t ld[kRN];        // P2-P3: claimed landing edges
-      uint16_t lv[kRN];        // P1-P2: unaligned marker list
-    } p;
+    uint16_t mk[kMkCap];       // P1-P3: region index of every marker, by rank
     struct {
       Cand cand[CAP];          // P4-P6
       int16_t next[CAP];       // candidate links
       uint16_t le[CAP];        // P5-P6: unaligned edges with a linked candidate
     } c;
   } u;
-  R hfx[kRN];              // moved aligned marker: fraction
-  R vfx[kRN];              // moved unaligned marker: fraction along the sweep (the one
-                           // across it is the marker's own, read from the state)
+  R fr[kMkCap];            // moved markers' fraction along the sweep, by rank (an unaligned
+                           // marker's one across it is its own, read from the state)
   alignas(16) uint32_t head[kNVE * head_bits<CAP>() / 32];  // first linked candidate of
                                                             // unaligned edges
                                         // 4m .. 4m+3 (8 bits each, 0xff: none)
   uint32_t kb[kRB];        // old corner colours
   uint32_t kn[kRB];        // new corner colours
   uint32_t zb[kRB];        // old centre colours (bit lx of row ly: cell (lx, ly))
-  union {
-    uint32_t hm[kRB];      // P1-P3: aligned markers (bit lx of row ly: edge (lx, ly))
-    uint32_t hc[kRB];      // P4-P6: unaligned edges with a linked candidate
-  };
-  union {
-    uint32_t vm[kRB];      // P1-P3: unaligned markers
-    uint32_t ovf[kRB];     // P4-P6: unaligned edges done in place
-  };
+  uint32_t hm[kRB];        // aligned markers (bit lx of row ly: edge (lx, ly))
+  uint32_t vm[kRB];        // unaligned markers
+  uint16_t hbase[kRB];     // rank of the first marker of each word
+  uint16_t vbase[kRB];
   uint32_t claim[kRB];     // aligned edges some marker lands on
+  uint32_t hc[kRB];        // unaligned edges with a linked candidate
+  uint32_t ovf[kRB];       // unaligned edges done in place
   // 2-bit codes (planes 0 and 1): moved aligned / unaligned marker ix - x + 1,
   // landing kept source - i + 2 (0: none)
   uint32_t hq[2][kRB];
   uint32_t vq[2][kRB];
   uint32_t lq[2][kRB];
   union {
-    uint16_t lh[kRN];      // P1-P2 aligned marker list; P3-P4 the interface-cell list
+    uint16_t cl[kMkCap];   // P3-P4: the segments (at most one per marker: a marker ends two)
     alignas(16) uint8_t vrl[kNVE];  // P5-P7: centre verdicts of an edge: bits 0-1
                                     // right + 1, bits 2-3 left + 1
   };
+  // Rank of the marker on aligned (kind 0) or unaligned edge (lx, ly): aligned
+  // ones first, each in region order.
+  __device__ __forceinline__ int rank(int kind, int lx, int ly) const {
+    const int w = ly * kRW + (lx >> 5);
+    const uint32_t below = (1u << (lx & 31)) - 1u;
+    return kind ? vbase[w] + __popc(vm[w] & below) : hbase[w] + __popc(hm[w] & below);
+  }
 };
 
 template <typename R, int CAP = kCandCap>
@@ -134,6 +144,15 @@ constexpr size_t tile_smem_bytes() {
 
 __device__ __forceinline__ int getb(const uint32_t* w, int lx, int ly) {
   return (w[ly * kRW + (lx >> 5)] >> (lx & 31)) & 1;
+}
+
+// Corner mask of region cell (lx, ly), counter-clockwise from its lower left
+// (lx < kRX - 1, so the word after the one of lx only counts within its row).
+__device__ __forceinline__ int corners4(const uint32_t* w, int lx, int ly) {
+  const uint32_t* q = w + ly * kRW + (lx >> 5);
+  const int lo = __funnelshift_r(q[0], q[1], lx & 31) & 3;
+  const int up = __funnelshift_r(q[kRW], q[kRW + 1], lx & 31) & 3;
+  return lo | ((up & 2) << 1) | ((up & 1) << 3);
 }
 
 // 2-bit code of region entry (lx, ly) held in two bit planes.
@@ -153,18 +172,6 @@ __device__ __forceinline__ uint32_t shr1(const uint32_t* w, int ly, int wi) {
   uint32_t v = w[ly * kRW + wi] >> 1;
   if (wi + 1 < kRW) v |= w[ly * kRW + wi + 1] << 31;
   return v;
-}
-
-// Appends the set bits of plane word t as region indices.
-__device__ __forceinline__ void push_bits(uint32_t bits, int t, uint16_t* list, int* count) {
-  if (!bits) return;
-  int base = atomicAdd(count, __popc(bits));
-  const int row0 = (t / kRW) * kRX + 32 * (t % kRW);
-  while (bits) {
-    const int b = __ffs(bits) - 1;
-    bits &= bits - 1;
-    list[base++] = (uint16_t)(row0 + b);
-  }
 }
 
 __device__ __forceinline__ int verdict_r(uint8_t c) { return (int)(c & 3) - 1; }
@@ -198,15 +205,17 @@ __device__ __forceinline__ void flush_count(int* s_cnt, int c, int v, int lane) 
   if (s != 0 && lane == 0) atomicAdd(&s_cnt[c], s);
 }
 
-// push_bits for a whole warp (all 32 lanes call it).
-__device__ __forceinline__ void push_bits_warp(uint32_t bits, int t, uint16_t* list, int* count,
-                                               int lane) {
+// Appends the set bits of plane word t as region indices (with flag), for a
+// whole warp (all 32 lanes call it).
+__device__ __forceinline__ void push_bits_warp(uint32_t bits, int t, int flag, uint16_t* list,
+                                               int* count, int lane) {
   int base = warp_alloc(__popc(bits), count, lane);
-  const int row0 = (t / kRW) * kRX + 32 * (t % kRW);
+  const int row0 = ((t / kRW) * kRX + 32 * (t % kRW)) | flag;
+#pragma unroll 1
   while (bits) {
     const int b = __ffs(bits) - 1;
     bits &= bits - 1;
-    list[base++] = (uint16_t)(row0 + b);
+    list[base++] = (uint16_t)(row0 + b);  // the flag bits lie above every region index
   }
 }
 
@@ -244,7 +253,7 @@ __device__ __forceinline__ uint32_t upto32(int c0, int last) {
 template <typename R, int AX, int LD, int CAP = kCandCap>
 struct TViewB {
   const TileMem<R, CAP>* m;
-  const GView<R, AX, LD>* g;  // an unaligned marker's own fraction is read from the state
+  GView<R, AX, LD> g;  // an unaligned marker's own fraction is read from the state
   int ri0, rj0, nx_, ny_;
   __device__ __forceinline__ int tnx() const { return nx_; }
   __device__ __forceinline__ int tny() const { return ny_; }
@@ -257,6 +266,7 @@ struct TViewB {
   __device__ __forceinline__ int k(int i, int j) const { return getb(m->kb, cx(i), cy(j)); }
   __device__ __forceinline__ int z(int i, int j) const { return getb(m->zb, cx(i), cy(j)); }
   __device__ __forceinline__ int knew(int i, int j) const { return getb(m->kn, cx(i), cy(j)); }
+  __device__ __forceinline__ int corners(int i, int j) const { return corners4(m->kb, cx(i), cy(j)); }
   __device__ __forceinline__ uint16_t ref(Mk mk) const {
     return (uint16_t)((cy(mk.j) * kRX + cx(mk.i)) | (mk.kind ? kKindV : 0));
   }
@@ -277,17 +287,16 @@ struct TViewB {
     return beyond(*this, n, ci, cj, &oi, &oj);
   }
   __device__ __forceinline__ AP<R> moved(Mk mk) const {
-    const int lx = cx(mk.i), ly = cy(mk.j), t = ly * kRX + lx;
+    const int lx = cx(mk.i), ly = cy(mk.j);
     AP<R> p;
     p.jy = mk.j;
+    p.fx = m->fr[m->rank(mk.kind, lx, ly)];
     if (mk.kind == 0) {
       p.ix = mk.i + get2(m->hq, lx, ly) - 1;
-      p.fx = m->hfx[t];
       p.fy = R(0);
     } else {
       p.ix = mk.i + get2(m->vq, lx, ly) - 1;
-      p.fx = m->vfx[t];
-      p.fy = g->v(mk.i, mk.j);
+      p.fy = g.v(mk.i, mk.j);
     }
     return p;
   }
@@ -307,10 +316,10 @@ struct TViewB {
     // the same values as (double)n + (double)f; the conversions run on the
     // integer pipe and an aligned marker's y needs no addition
     if (r & kKindV) {
-      *X = i2d(ri0 + lx + get2(m->vq, lx, ly) - 1 - k) + to_d<R>(m->vfx[t]);
-      *Y = i2d(rj0 + ly - j) + to_d<R>(g->v(ri0 + lx, rj0 + ly));
+      *X = i2d(ri0 + lx + get2(m->vq, lx, ly) - 1 - k) + to_d<R>(m->fr[m->rank(1, lx, ly)]);
+      *Y = i2d(rj0 + ly - j) + to_d<R>(g.v(ri0 + lx, rj0 + ly));
     } else {
-      *X = i2d(ri0 + lx + get2(m->hq, lx, ly) - 1 - k) + to_d<R>(m->hfx[t]);
+      *X = i2d(ri0 + lx + get2(m->hq, lx, ly) - 1 - k) + to_d<R>(m->fr[m->rank(0, lx, ly)]);
       *Y = i2d(rj0 + ly - j);
     }
   }
@@ -319,7 +328,7 @@ struct TViewB {
   __device__ __forceinline__ R own_fraction(uint16_t r) const {
     if (!(r & kKindV)) return R(0);
     const int t = r & (kKindV - 1), ly = t / kRX, lx = t - ly * kRX;
-    return g->v(ri0 + lx, rj0 + ly);
+    return g.v(ri0 + lx, rj0 + ly);
   }
   // The point in the FP32 form, given its own fraction fy: the exact sums by
   // integer operations where they are exact (add_nf), and a float estimate
@@ -332,11 +341,11 @@ struct TViewB {
     float fx;
     if (r & kKindV) {
       nx = ri0 + lx + get2(m->vq, lx, ly) - 1 - k;
-      fx = (float)m->vfx[t];
+      fx = (float)m->fr[m->rank(1, lx, ly)];
       *Y = add_nf(ny, fy);
     } else {
       nx = ri0 + lx + get2(m->hq, lx, ly) - 1 - k;
-      fx = (float)m->hfx[t];
+      fx = (float)m->fr[m->rank(0, lx, ly)];
       fy = 0.0f;
       *Y = i2d(ny);
     }
@@ -355,23 +364,7 @@ template <typename R, int CAP>
 __device__ __forceinline__ NewV<R> select_linked(const TileMem<R, CAP>& M, int s, int present,
                                                  int* kept) {
   *kept = -1;
-  if (s >= 0 && M.u.c.next[s] < 0 && present) {
-    // one candidate on an edge that keeps a marker: it is the marker (the
-    // common case, without the ranking below)
-    const Cand& C = M.u.c.cand[s];
-    NewV<R> one;
-    *kept = s;
-    one.present = 1;
-    one.vr = -1;
-    one.vl = -1;
-    one.cancelled = 0;
-    one.invariant = 0;
-    if constexpr (sizeof(R) == 4) one.s = C.sf;
-    else one.s = to_fraction<R>(C.y);
-    return one;
-  }
   double cy[6];
-  float sf[6];
   long long key[6];
   int ord[6], sl[6];
   int n = 0;
@@ -380,7 +373,6 @@ __device__ __forceinline__ NewV<R> select_linked(const TileMem<R, CAP>& M, int s
     if (s >= 0) {
       const Cand& C = M.u.c.cand[s];
       cy[q] = C.y;
-      sf[q] = C.sf;
       key[q] = okey(C.y);
       ord[q] = C.ord;
       sl[q] = s;
@@ -388,7 +380,6 @@ __device__ __forceinline__ NewV<R> select_linked(const TileMem<R, CAP>& M, int s
       s = M.u.c.next[s];
     } else {
       cy[q] = 0.0;
-      sf[q] = 0.0f;
       key[q] = 0;
       ord[q] = 0;
       sl[q] = -1;
@@ -433,22 +424,177 @@ __device__ __forceinline__ NewV<R> select_linked(const TileMem<R, CAP>& M, int s
   }
   if (want >= 0) {
     double ysel = 0.0;
-    float fsel = 0.0f;
 #pragma unroll
     for (int t = 0; t < 6; ++t)
       if (t < n && rank[t] == want) {
         ysel = cy[t];
-        fsel = sf[t];
         *kept = sl[t];
       }
-    if constexpr (sizeof(R) == 4) out.s = fsel;  // to_fraction<float>, taken in the fit phase
-    else out.s = to_fraction<R>(ysel);
+    out.s = to_fraction<R>(ysel);
   }
   return out;
 }
 
-// The tile with origin (i0, j0) of one grid (one block runs it).
-template <typename R, int AX, int LD, int CAP = kCandCap>
+// The parts of the tile that few tiles or few markers take are kept out of
+// line, with their loops rolled: inlined they made the kernel 390 KB of code,
+// three times the instruction cache.
+
+// Landings on one edge other than a single one that stays.
+template <typename R>
+__device__ __noinline__ Landing<R> landing_rare(bool v0, bool v1, bool v2, R f0, R f1, R f2, int x, int present) {
+  const bool valid[3] = {v0, v1, v2};
+  const R fx[3] = {f0, f1, f2};
+  return choose_landing3<R>(valid, fx, x, present);
+}
+
+// One marker of an edge with several candidates (or none to keep): see
+// select_linked.
+template <typename R, int CAP>
+__device__ __noinline__ NewV<R> select_rare(const TileMem<R, CAP>& M, int s, int present, int* kept) {
+  return select_linked<R>(M, s, present, kept);
+}
+
+// The marker beyond point 1 (side 0) or 4 (side 1) of a candidate, as a third
+// point for its ends (ax, ay) and (bx, by).
+struct NextPt {
+  FitPt T;
+  bool found;
+};
+template <typename R, int AX, int LD, int CAP>
+__device__ __noinline__ NextPt next_point(const TViewB<R, AX, LD, CAP> TV, int slot, int side, int k, int j,
+                                          double ax, double ay, double bx, double by) {
+  NextPt p{};
+  const Mk q = TV.next_beyond(TV.m->u.c.cand[slot], side, k, j);
+  p.found = q.kind >= 0;
+  if (p.found) {
+    double X, Y;
+    TV.xy(TV.ref(q), k, j, &X, &Y);
+    p.T = fit_pt(X, Y, ax, ay, bx, by);
+  }
+  return p;
+}
+
+// Centre-rule verdicts (right + 1, left + 1 as in verdicts()) of the kept
+// candidate of unaligned edge (k, j), for the sides asked for.
+template <typename R, int AX, int LD, int CAP>
+__device__ __noinline__ uint8_t verdicts_of(const TViewB<R, AX, LD, CAP> TV, int slot, int k, bool right, bool left) {
+  const Cand& C = TV.m->u.c.cand[slot];
+  int v[2] = {-1, -1};
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    if (!(side ? left : right)) continue;
+    const Mk none{-1, 0, 0};
+    const Mk far = (C.fl & (side ? CF_P1 : CF_P4)) ? TV.mk(side ? C.p1 : C.p4) : none;
+    const int line = walk(TV, TV.mk(side ? C.a : C.b), far, side ? k - 1 : k);
+    if (line >= 0) v[side] = !TV.knew(k, line);
+  }
+  return verdicts(v[0], v[1]);
+}
+
+// new_unaligned out of line.
+template <typename R, class A>
+__device__ __noinline__ NewV<R> new_unaligned_rare(const A S, bool line_only, int k, int j, int* cnt) {
+  return new_unaligned<R>(S, line_only, k, j, cnt);
+}
+
+// The tile with origin (i0, j0) by the generic logic, every answer recomputed
+// from global memory: for the tiles whose region holds more markers than
+// shared memory keeps (over a quarter of its edges, as noise does), so that
+// any state is swept.
+template <typename R, int AX, int LD, int T>
+__device__ __noinline__ void tile_in_place(const GView<R, AX, LD> G, const Buf<R> out, int line_only,
+                                           unsigned long long* ctr, unsigned long long* cfl_bits,
+                                           int* status, const int i0, const int j0) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tnx = G.tnx(), tny = G.tny();
+  const long long P = G.d.P;
+  int cnt[D_NUSED];
+#pragma unroll 1
+  for (int c = 0; c < D_NUSED; ++c) cnt[c] = 0;
+  double dmax = 0.0;
+  // a warp takes 32 vertices that share a stored colour word
+#pragma unroll 1
+  for (int q = warp; q < 2 * kTJ; q += T / 32) {
+    const int i = AX ? i0 + q : i0 + 32 * (q & 1) + lane;
+    const int j = AX ? j0 + lane : j0 + (q >> 1);
+    const bool vertex = i <= tnx && j <= tny, cell = i < tnx && j < tny;
+    int kn = 0, zn = 0;
+    Flags f;
+    if (vertex) kn = G.knew(i, j);
+    if (i < tnx && j <= tny) {  // aligned edge
+      if (G.k(i, j) != G.k(i + 1, j)) {
+        G.advect(Mk{0, i, j}, f);
+        cnt[D_CFL] += f.cfl;
+        cnt[D_WALL_CLAMP] += f.clamp;
+      }
+      const Landing<R> L = G.landing(i, j);
+      cnt[D_CANCELLED] += L.cancelled;
+      cnt[D_INVARIANT] += L.invariant;
+      if (L.present) {
+        if (AX) { if (in_range((long long)i * P + j, G.d.nV())) out.sV[(long long)i * P + j] = L.kept_fx; }
+        else if (in_range((long long)j * P + i, G.d.nH())) out.sH[(long long)j * P + i] = L.kept_fx;
+      }
+    }
+    if (i <= tnx && j < tny) {  // unaligned edge
+      const bool inner = i >= 1 && i <= tnx - 1, old = G.k(i, j) != G.k(i, j + 1);
+      R s = R(0);
+      bool put = false;
+      if (inner && old) {
+        Flags g;
+        G.advect(Mk{1, i, j}, g);
+        cnt[D_CFL] += g.cfl;
+        f.dabs = fmaxf(f.dabs, g.dabs);
+        f.dabs64 = fmax(f.dabs64, g.dabs64);
+      }
+      if (inner) {
+        const NewV<R> nv = new_unaligned_rare<R>(G, line_only != 0, i, j, cnt);
+        put = nv.present != 0;
+        s = nv.s;
+      } else if (old) {  // a wall marker normal to the sweep stays
+        put = true;
+        s = G.v(i, j);
+      }
+      if (put) {
+        if (AX) { if (in_range((long long)i * P + j, G.d.nH())) out.sH[(long long)i * P + j] = s; }
+        else if (in_range((long long)j * P + i, G.d.nV())) out.sV[(long long)j * P + i] = s;
+      }
+    }
+    if (cell) {
+      zn = G.z(i, j);
+      const int a = kn, b = G.knew(i + 1, j), c = G.knew(i + 1, j + 1), d = G.knew(i, j + 1);
+      if (a != b && b != c && c != d) {  // four markers: the verdicts of its unaligned edges
+        const int vr = i >= 1 ? new_unaligned_rare<R>(G, line_only != 0, i, j, nullptr).vr : -1;
+        const int vl = i + 1 <= tnx - 1 ? new_unaligned_rare<R>(G, line_only != 0, i + 1, j, nullptr).vl : -1;
+        if (vr >= 0 || vl >= 0) {
+          cnt[D_ZSET] += 1;
+          cnt[D_ZCONFLICT] += vr >= 0 && vl >= 0 && vr != vl;
+          zn = vr >= 0 ? vr : vl;
+        }
+      }
+    }
+    dmax = fmax(dmax, (double)dabs_of<R>(f));
+    const uint32_t kw = __ballot_sync(kFull, kn != 0), zw = __ballot_sync(kFull, zn != 0);
+    const int row = AX ? i : j, word = (AX ? j0 : i0 + 32 * (q & 1)) >> 5;
+    if (lane == 0) {
+      if (row <= G.d.ny && word < G.d.kw) out.K[(long long)row * G.d.kw + word] = kw;
+      if (row < G.d.ny && word < G.d.zw) out.Z[(long long)row * G.d.zw + word] = zw;
+    }
+  }
+#pragma unroll 1
+  for (int c = 0; c < D_NUSED; ++c) {
+    const int s = __reduce_add_sync(kFull, cnt[c]);
+    if (s == 0 || lane != 0) continue;
+    atomicAdd(&ctr[c], (unsigned long long)s);
+    if (c == D_CFL) atomicOr(status, ST_CFL);
+    if (c == D_INVARIANT) atomicOr(status, ST_INVARIANT);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) dmax = fmax(dmax, __shfl_xor_sync(kFull, dmax, o));
+  if (lane == 0 && dmax > 0.0) atomicMax(cfl_bits, (unsigned long long)__double_as_longlong(dmax));
+}
+
+// The tile with origin (i0, j0) of one grid (one block of T threads runs it).
+template <typename R, int AX, int LD, int CAP = kCandCap, int T = tile_threads<R>()>
 __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<R>& out, int line_only,
                                            unsigned long long* ctr, unsigned long long* cfl_bits,
                                            int* status, const int i0, const int j0) {
@@ -456,19 +602,19 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
   TileMem<R, CAP>& M = *reinterpret_cast<TileMem<R, CAP>*>(smem_raw);
   constexpr int kHB = head_bits<CAP>(), kHPW = 32 / kHB;  // head bits, heads per word
   constexpr uint32_t kHNone = head_none<CAP>();
-  __shared__ int s_nh, s_nv, s_nd, s_nc, s_ncand, s_ne, s_novf;
+  __shared__ int s_nh, s_nm, s_nc, s_ncand, s_ne, s_novf;
   __shared__ int s_cnt[D_NUSED];
   __shared__ unsigned long long s_dmax;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kTileThreads = tile_threads<R>();
+  constexpr int kTileThreads = T;
   constexpr int kWarps = kTileThreads / 32;
   const int tnx = G.tnx(), tny = G.tny();
   const int ri0 = i0 - 4, rj0 = j0 - 2;
   const long long P = G.d.P;
   if (tid < D_NUSED) s_cnt[tid] = 0;
   if (tid == 0) {
-    s_nh = s_nv = s_nd = s_nc = s_ncand = s_ne = s_novf = 0;
+    s_nc = s_ncand = s_ne = s_novf = 0;
     s_dmax = 0ull;
   }
   auto owned = [&](int x, int y) { return x >= i0 && x < i0 + kTI && y >= j0 && y < j0 + kTJ; };
@@ -481,7 +627,8 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
 
   // P0: colour bits of the region
   if (AX == 0) {
-    for (int t = tid; t < 2 * kRB; t += kTileThreads) {
+  #pragma unroll 1
+  for (int t = tid; t < 2 * kRB; t += kTileThreads) {
       const int zpl = t >= kRB, u = zpl ? t - kRB : t;
       const int ly = u / kRW, wi = u % kRW;
       const int y = rj0 + ly, x0 = ri0 + 32 * wi;
@@ -531,6 +678,8 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
     M.vm[t] = v;
     M.kn[t] = M.kb[t];
     M.claim[t] = 0u;
+    M.hc[t] = 0u;
+    M.ovf[t] = 0u;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       M.hq[q][t] = 0u;
@@ -540,13 +689,43 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
     mine |= (h | v) != 0u;
   }
   const bool busy = __syncthreads_or(mine) != 0;
-  const TViewB<R, AX, LD, CAP> TV{&M, &G, ri0, rj0, tnx, tny};
+  const TViewB<R, AX, LD, CAP> TV{&M, G, ri0, rj0, tnx, tny};
 
   if (busy) {
-    for (int t0 = warp * 32; t0 < kRB; t0 += kTileThreads) {
-      const int t = t0 + lane;
-      push_bits_warp(t < kRB ? M.hm[t] : 0u, t, M.lh, &s_nh, lane);
-      push_bits_warp(t < kRB ? M.vm[t] : 0u, t, M.u.p.lv, &s_nv, lane);
+    // ranks: warps 0 and 1 take the halves of the aligned set's words, warps 2
+    // and 3 those of the unaligned set, two words a lane; the markers before a
+    // warp's first word are counted by the warp itself
+    static_assert(kWarps >= 4 && kRB <= 128, "two words a lane, two warps a set");
+    if (warp < 4) {
+      const int pl = warp >> 1, hf = warp & 1, t0 = 64 * hf + 2 * lane;
+      const uint32_t* pm = pl ? M.vm : M.hm;
+      uint32_t w0 = t0 < kRB ? pm[t0] : 0u, w1 = t0 + 1 < kRB ? pm[t0 + 1] : 0u;
+      const int n0 = __popc(w0), n = n0 + __popc(w1);
+      int before = 0;
+      if (hf) before = __popc(pm[lane]) + __popc(pm[lane + 32]);
+      if (pl) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (lane + 32 * q < kRB) before += __popc(M.hm[lane + 32 * q]);
+      }
+      before = __reduce_add_sync(kFull, before);
+      int incl = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += v;
+      }
+      int at = before + incl - n;
+      uint16_t* base = pl ? M.vbase : M.hbase;
+      if (t0 < kRB) base[t0] = (uint16_t)at;
+      if (t0 + 1 < kRB) base[t0 + 1] = (uint16_t)(at + n0);
+      if (hf && lane == 31) (pl ? s_nm : s_nh) = at + n;
+      const int r0 = (t0 / kRW) * kRX + 32 * (t0 % kRW);
+      const int r1 = ((t0 + 1) / kRW) * kRX + 32 * ((t0 + 1) % kRW);
+#pragma unroll 1
+      for (; w0 && at < kMkCap; w0 &= w0 - 1) M.u.mk[at++] = (uint16_t)(r0 + __ffs(w0) - 1);
+#pragma unroll 1
+      for (; w1 && at < kMkCap; w1 &= w1 - 1) M.u.mk[at++] = (uint16_t)(r1 + __ffs(w1) - 1);
     }
     static_assert(sizeof(M.head) % 16 == 0, "vector initialisation");
     for (int e = tid; e < (int)(sizeof(M.head) / 16); e += kTileThreads)
@@ -555,56 +734,39 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
 
     // P2: moved points (aligned and unaligned markers in one pass), corner
     // flips, landing claims
-    const int nh = s_nh, nm = s_nh + s_nv;
+    const int nh = s_nh, nm = s_nm;
+    if (nm > kMkCap) {  // the same in every thread
+      tile_in_place<R, AX, LD, T>(G, out, line_only, ctr, cfl_bits, status, i0, j0);
+      return;
+    }
     int n_cfl = 0, n_clamp = 0;
     R dmax = R(0);
-    for (int w0 = warp * 32; w0 < nm; w0 += kTileThreads) {
-      const int w = w0 + lane;
-      int claimed = -1;
-      if (w < nh) {
-        const int id = M.lh[w], lx = id % kRX, ly = id / kRX;
-        const int x = ri0 + lx, y = rj0 + ly;
-        Flags f;
-        const AP<R> p = G.advect(Mk{0, x, y}, f);
-        put2(M.hq, lx, ly, p.ix - x + 1);
-        M.hfx[id] = p.fx;
-        if (owned(x, y)) {
-          n_cfl += f.cfl;
-          n_clamp += f.clamp;
-          dmax = fmax(dmax, dabs_of<R>(f));
-        }
-        // a marker moving right passes vertex x+1, one moving left vertex x
-        if (p.ix == x + 1) atomicXor(&M.kn[ly * kRW + ((lx + 1) >> 5)], 1u << ((lx + 1) & 31));
-        else if (p.ix == x - 1) atomicXor(&M.kn[ly * kRW + (lx >> 5)], 1u << (lx & 31));
-        const int dl = p.ix - ri0;
-        if (dl >= 1 && dl <= kRX - 3) {
-          const uint32_t bit = 1u << (dl & 31);
-          if (!(atomicOr(&M.claim[ly * kRW + (dl >> 5)], bit) & bit)) claimed = ly * kRX + dl;
-        }
-      } else if (w < nm) {
-        const int id = M.u.p.lv[w - nh], lx = id % kRX, ly = id / kRX;
-        const int x = ri0 + lx, y = rj0 + ly;
-        Flags f;
-        const AP<R> p = G.advect(Mk{1, x, y}, f);
-        put2(M.vq, lx, ly, p.ix - x + 1);
-        M.vfx[id] = p.fx;
-        if (owned(x, y)) {
-          if (x >= 1 && x <= tnx - 1) {
-            n_cfl += f.cfl;
-            dmax = fmax(dmax, dabs_of<R>(f));
-          } else {  // a wall marker normal to the sweep stays
-            if (AX) { if (in_range((long long)x * P + y, G.d.nH())) out.sH[(long long)x * P + y] = p.fy; }
-            else if (in_range((long long)y * P + x, G.d.nV())) out.sV[(long long)y * P + x] = p.fy;
-          }
-        }
+#pragma unroll 1
+    for (int w = tid; w < nm; w += kTileThreads) {
+      const int id = M.u.mk[w], lx = id % kRX, ly = id / kRX;
+      const int x = ri0 + lx, y = rj0 + ly;
+      const bool al = w < nh;
+      Flags f;
+      const AP<R> p = G.advect(Mk{al ? 0 : 1, x, y}, f);
+      M.fr[w] = p.fx;
+      put2(al ? M.hq : M.vq, lx, ly, p.ix - x + 1);
+      const bool own = owned(x, y);
+      if (own) {  // no flag on a wall normal to the sweep
+        n_cfl += f.cfl;
+        n_clamp += f.clamp;
+        dmax = fmax(dmax, dabs_of<R>(f));
       }
-      const unsigned cm = __ballot_sync(kFull, claimed >= 0);
-      if (cm) {
-        const int leader = __ffs(cm) - 1;
-        int base = 0;
-        if (lane == leader) base = atomicAdd(&s_nd, __popc(cm));
-        base = __shfl_sync(kFull, base, leader);
-        if (claimed >= 0) M.u.p.ld[base + __popc(cm & ((1u << lane) - 1u))] = (uint16_t)claimed;
+      if (al) {
+        // a marker moving right passes vertex x+1, one moving left vertex x
+        if (p.ix != x) {
+          const int c = lx + (p.ix > x);
+          atomicXor(&M.kn[ly * kRW + (c >> 5)], 1u << (c & 31));
+        }
+        const int dl = p.ix - ri0;
+        if (dl >= 1 && dl <= kRX - 3) atomicOr(&M.claim[ly * kRW + (dl >> 5)], 1u << (dl & 31));
+      } else if (own && (x == 0 || x == tnx)) {  // a wall marker normal to the sweep stays
+        if (AX) { if (in_range((long long)x * P + y, G.d.nH())) out.sH[(long long)x * P + y] = p.fy; }
+        else if (in_range((long long)y * P + x, G.d.nV())) out.sV[(long long)y * P + x] = p.fy;
       }
     }
     flush_count(s_cnt, D_CFL, n_cfl, lane);
@@ -615,26 +777,35 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       atomicMax(&s_dmax, (unsigned long long)__double_as_longlong((double)dmax));
     __syncthreads();
 
-    // P3: landings on the claimed aligned edges
-    // landings on warps 0-4, the word pass (owned edges without a landing,
-    // interface cells) on warps 5-7 at the same time
-    const int nd = s_nd;
+    // P3: landings.  Of the markers landing on an edge the one from the lowest
+    // source takes the edge.  The word pass (owned edges without a landing,
+    // interface cells) is the last three warps', which join the landings
+    // after it.
     int n_canc = 0, n_inv = 0;
     constexpr int kSplit = kTileThreads - kTJ * kRW;  // 96 words on the last three warps
     static_assert(kSplit > 0 && kSplit % 32 == 0, "warp split");
-    for (int w = tid; w < nd && tid < kSplit; w += kSplit) {
-      const int id = M.u.p.ld[w], dl = id % kRX, ly = id / kRX;
+#pragma unroll 1
+    for (int w = tid; w < nh; w += kTileThreads) {
+      const int id = M.u.mk[w], lx = id % kRX, ly = id / kRX;
+      const int dl = lx + get2(M.hq, lx, ly) - 1;
+      if (dl < 1 || dl > kRX - 3) continue;
       const int x = ri0 + dl, y = rj0 + ly;
       bool valid[3];
       R fx[3];
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        const int e = dl - 1 + q, ie = ly * kRX + e;
+        const int e = dl - 1 + q;
         valid[q] = getb(M.hm, e, ly) && e + get2(M.hq, e, ly) - 1 == dl;
-        fx[q] = valid[q] ? M.hfx[ie] : R(0);
+        fx[q] = valid[q] ? M.fr[M.rank(0, e, ly)] : R(0);
       }
-      const Landing<R> L =
-          choose_landing3<R>(valid, fx, x, getb(M.kn, dl, ly) ^ getb(M.kn, dl + 1, ly));
+      if (lx != dl - 1 && (valid[0] || (lx != dl && valid[1]))) continue;  // a lower source's edge
+      const int present = getb(M.kn, dl, ly) ^ getb(M.kn, dl + 1, ly);
+      Landing<R> L;
+      if (present && (int)valid[0] + (int)valid[1] + (int)valid[2] == 1) {  // it stays
+        L = Landing<R>{1, ri0 + lx, 0, 0, M.fr[w]};
+      } else {
+        L = landing_rare<R>(valid[0], valid[1], valid[2], fx[0], fx[1], fx[2], x, present);
+      }
       if (L.kept_src >= 0) put2(M.lq, dl, ly, L.kept_src - x + 2);
       if (owned(x, y)) {
         n_canc += L.cancelled;
@@ -653,6 +824,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       if (ly <= vy1) {
         uint32_t bad = (M.kn[u] ^ shr1(M.kn, ly, wi)) & ~M.claim[u] &
                        span_mask(wi, 4, min(kTI + 3, ex1));
+#pragma unroll 1
         while (bad) {
           const int b = __ffs(bad) - 1;
           bad &= bad - 1;
@@ -664,95 +836,94 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       }
       // interface cells (corner colours not all equal) whose chords can
       // cross a grid line k in [i0, i0+64]: cells k-2..k
-      uint32_t ic = 0u;
+      uint32_t ic = 0u, four = 0u;
       if (ly <= ty1) {
-        const uint32_t a = M.kb[u], b = M.kb[u + kRW];
-        ic = ((a ^ shr1(M.kb, ly, wi)) | (b ^ shr1(M.kb, ly + 1, wi)) | (a ^ b)) &
-             span_mask(wi, max(2, vx0), min(kTI + 4, ex1));
+        const uint32_t a = M.kb[u], b = M.kb[u + kRW], a1 = shr1(M.kb, ly, wi), b1 = shr1(M.kb, ly + 1, wi);
+        const uint32_t cm = span_mask(wi, max(2, vx0), min(kTI + 4, ex1));
+        ic = ((a ^ a1) | (b ^ b1) | (a ^ b)) & cm;
+        four = (a ^ a1) & (b ^ b1) & (a ^ b) & cm;
       }
-      push_bits_warp(ic, u, M.lh, &s_nc, lane);
+      push_bits_warp(ic, u, 0, M.cl, &s_nc, lane);
+      if (__any_sync(kFull, four != 0u)) push_bits_warp(four, u, kSecond, M.cl, &s_nc, lane);
     }
     flush_count(s_cnt, D_CANCELLED, n_canc, lane);
     flush_count(s_cnt, D_INVARIANT, n_inv, lane);
     __syncthreads();
-    // the marker sets are dead: their storage becomes the candidate sets
-    for (int t = tid; t < kRB; t += kTileThreads) {
-      M.hc[t] = 0u;
-      M.ovf[t] = 0u;
-    }
-    __syncthreads();
 
-    // P4: candidates.  A thread takes one interface cell: counts the grid
-    // lines its moved chords cross, takes that many slots, then fills them.
+    // P4: candidates.  A thread takes one segment: counts the grid lines its
+    // moved chord crosses, takes that many slots, then fills them.
     const int nc = s_nc;
     const int kmin = max(1, i0), kmax = min(tnx - 1, i0 + kTI);
+#pragma unroll 1
     for (int w0 = warp * 32; w0 < nc; w0 += kTileThreads) {
       const int w = w0 + lane;
-      int c = 0, j = 0, ly = 0, ns = 0, ncross = 0;
-      int seg[2][2] = {{0, 0}, {0, 0}};
-      int ia[2] = {0, 0}, ib[2] = {0, 0};
+      int lx = 0, ly = 0, second = 0, ea = 0, eb = 0, xa = 0, klo = 0, khi = -1;
+      // edge e of the cell as a region index
+      auto at = [&](int e) { return (ly + (e == 2)) * kRX + lx + (e == 1); };
       if (w < nc) {
-        const int id = M.lh[w], lx = id % kRX;
-        ly = id / kRX;
-        c = ri0 + lx;
-        j = rj0 + ly;
-        ns = cell_segments(TV, c, j, seg);
-#pragma unroll
-        for (int t = 0; t < 2; ++t)
-          if (t < ns) {
-            ia[t] = TV.moved(edge_marker(c, j, seg[t][0])).ix;
-            ib[t] = TV.moved(edge_marker(c, j, seg[t][1])).ix;
-            ncross += max(0, min(max(ia[t], ib[t]), kmax) - max(min(ia[t], ib[t]) + 1, kmin) + 1);
-          }
-      }
-      int slot = warp_alloc(ncross, &s_ncand, lane);
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        if (t >= ns) continue;
-        const Mk ma = edge_marker(c, j, seg[t][0]);
-        const Mk mb = edge_marker(c, j, seg[t][1]);
-        const int klo = max(min(ia[t], ib[t]) + 1, kmin), khi = min(max(ia[t], ib[t]), kmax);
-        for (int k = klo; k <= khi; ++k, ++slot) {
-          const int e = (j - j0) * (kTI + 1) + (k - i0);
-          const int ex = k - ri0, eu = ly * kRW + (ex >> 5);
-          const uint32_t ebit = 1u << (ex & 31);
-          if (slot >= CAP) {
-            atomicOr(&M.ovf[eu], ebit);
-            continue;
-          }
-          const bool a_left = ia[t] < k;
-          const Mk mA = a_left ? ma : mb, mB = a_left ? mb : ma;
-          Cand& C = M.u.c.cand[slot];
-          C.a = TV.ref(mA);
-          C.b = TV.ref(mB);
-          uint8_t fl = k < i0 + kTI ? CF_OWNED : 0;
-          int c1i = 0, c1j = 0, c4i = 0, c4j = 0;
-          const Mk n1 = beyond(TV, mA, c, j, &c1i, &c1j);
-          const Mk n4 = beyond(TV, mB, c, j, &c4i, &c4j);
-          if (n1.kind >= 0) {
-            C.p1 = TV.ref(n1);
-            fl |= CF_P1;
-          }
-          if (n4.kind >= 0) {
-            C.p4 = TV.ref(n4);
-            fl |= CF_P4;
-          }
-          C.fl = fl;
-          C.edge = (uint16_t)e;
-          C.ord = (uint8_t)((c - (k - 2)) * 2 + t);
-          {  // push the slot on the edge's list: a head of kHB bits in a shared word
-            uint32_t* hw = &M.head[e / kHPW];
-            const int sh = (e % kHPW) * kHB;
-            uint32_t old = *hw, seen;
-            do {  // each retry follows another thread's successful update
-              seen = old;
-              old = atomicCAS(hw, seen, (seen & ~(kHNone << sh)) | ((uint32_t)slot << sh));
-            } while (old != seen);
-            const uint32_t prev = (seen >> sh) & kHNone;
-            M.u.c.next[slot] = prev == kHNone ? (int16_t)-1 : (int16_t)prev;
-          }
-          atomicOr(&M.hc[eu], ebit);
+        const int id = M.cl[w], cell = id & (kSecond - 1);
+        second = id >= kSecond;
+        ly = cell / kRX;
+        lx = cell - ly * kRX;
+        const int q = corners4(M.kb, lx, ly), em = edge_mask(q);
+        ea = __ffs(em) - 1;
+        eb = 31 - __clz(em);
+        if (em == 15) {  // the pairs of segments()
+          const bool same = (q & 1) == getb(M.zb, lx, ly);
+          ea = same ? 2 * second : 3 - 2 * second;
+          eb = same ? ea + 1 : 2 * second;
         }
+        auto line = [&](int e) {
+          return ri0 + lx + (e == 1) + get2(e & 1 ? M.vq : M.hq, lx + (e == 1), ly + (e == 2)) - 1;
+        };
+        xa = line(ea);
+        const int xb = line(eb);
+        klo = max(min(xa, xb) + 1, kmin);
+        khi = min(max(xa, xb), kmax);
+      }
+      int slot = warp_alloc(max(0, khi - klo + 1), &s_ncand, lane);
+#pragma unroll 1
+      for (int k = klo; k <= khi; ++k, ++slot) {
+        const int j = rj0 + ly, e = (j - j0) * (kTI + 1) + (k - i0);
+        const int ex = k - ri0, eu = ly * kRW + (ex >> 5);
+        const uint32_t ebit = 1u << (ex & 31);
+        if (slot >= CAP) {
+          atomicOr(&M.ovf[eu], ebit);
+          continue;
+        }
+        Cand& C = M.u.c.cand[slot];
+        uint8_t fl = k < i0 + kTI ? CF_OWNED : 0;
+        // sides A (left of the line) and B: the chord's end, and the marker
+        // beyond it (point 1, 4) in the cell across the end's edge
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+          const int se = (xa < k) == (side == 0) ? ea : eb;
+          (side ? C.b : C.a) = (uint16_t)(at(se) | (se & 1 ? kKindV : 0));
+          const int ox = lx + (se == 1) - (se == 3), oy = ly + (se == 2) - (se == 0);
+          if ((unsigned)(ri0 + ox) < (unsigned)tnx && (unsigned)(rj0 + oy) < (unsigned)tny) {
+            const int q = corners4(M.kb, ox, oy), em = edge_mask(q), in = se ^ 2;
+            int pe = __ffs(em & ~(1 << in)) - 1;  // partner()
+            if (em == 15) pe = (q & 1) == getb(M.zb, ox, oy) ? in ^ 1 : 3 - in;
+            (side ? C.p4 : C.p1) =
+                (uint16_t)(((oy + (pe == 2)) * kRX + ox + (pe == 1)) | (pe & 1 ? kKindV : 0));
+            fl |= side ? CF_P4 : CF_P1;
+          }
+        }
+        C.fl = fl;
+        C.edge = (uint16_t)e;
+        C.ord = (uint8_t)((ri0 + lx - (k - 2)) * 2 + second);
+        {  // push the slot on the edge's list: a head of kHB bits in a shared word
+          uint32_t* hw = &M.head[e / kHPW];
+          const int sh = (e % kHPW) * kHB;
+          uint32_t old = *hw, seen;
+          do {  // each retry follows another thread's successful update
+            seen = old;
+            old = atomicCAS(hw, seen, (seen & ~(kHNone << sh)) | ((uint32_t)slot << sh));
+          } while (old != seen);
+          const uint32_t prev = (seen >> sh) & kHNone;
+          M.u.c.next[slot] = prev == kHNone ? (int16_t)-1 : (int16_t)prev;
+        }
+        atomicOr(&M.hc[eu], ebit);
       }
     }
     __syncthreads();
@@ -769,13 +940,14 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
     if (warp >= kWarps - 3) {
       const int t = (warp - (kWarps - 3)) * 32 + lane;  // kTJ * kRW = 96 words
       const int u = (2 + t / kRW) * kRW + t % kRW;
-      push_bits_warp(M.hc[u], u, M.u.c.le, &s_ne, lane);
+      push_bits_warp(M.hc[u], u, 0, M.u.c.le, &s_ne, lane);
       const int no = __reduce_add_sync(kFull, __popc(M.ovf[u]));  // edges done in place
       if (no != 0 && lane == 0) atomicAdd(&s_novf, no);
     }
     const int rot = (int)((blockIdx.x + blockIdx.y) & 3u);
     int n_fit[4] = {0, 0, 0, 0};  // D_FIT_ONLINE .. D_FIT_TWO
     const int vt = (((warp + rot) % kWarps) << 5) | lane;
+#pragma unroll 1
     for (int b0 = 0; b0 < 2 * ncand; b0 += kTileThreads) {
       const int item = b0 + vt, side = item & 1;
       Cand& C = M.u.c.cand[min(item >> 1, CAP - 1)];
@@ -813,61 +985,50 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       const double c2 = side ? osq + sq : sq + osq;  // cx*cx + cy*cy
       const double x0 = -ax;
       const bool online = d_eq0(bx);
+      // the third point, then the circle.  The warp's lanes come together
+      // between the two, so that those whose point takes longer do not run
+      // the circle's FP64 chain a second time.
       double ys = 0.0;
       bool ok = false;
-      if (act && !online) {
-        const uint8_t fl = C.fl;
-        if (!line_only && !d_below_sep(c2) && (fl & (side ? CF_P4 : CF_P1))) {
-          if constexpr (sizeof(R) == 4) {
-            // the third point's offsets from A exactly; its distance from B
-            // only where a float estimate (error below 2e-6 per component)
-            // does not already put it clearly past the minimum separation
-            double rx, ry, r2;
-            bool tfar;
-            auto third = [&](uint16_t ref, float fy) {
-              double X, Y;
-              float Xf, Yf;
-              TV.xyf(ref, k, j, fy, &X, &Y, &Xf, &Yf);
-              rx = X - ax;
-              ry = Y - ay;
-              r2 = rx * rx + ry * ry;
-              const float txf = Xf - bxf, tyf = Yf - byf;
-              if (txf * txf + tyf * tyf >= 1.5e-4f) {
-                tfar = true;
-              } else {
-                const double tx = X - bx, ty = Y - by;
-                tfar = !d_below_sep(tx * tx + ty * ty);
-              }
-            };
-            third(side ? C.p4 : C.p1, fy_t);
-            bool use = true;
-            if (side ? !tfar : d_below_sep(r2)) {  // too close to B (A): the next marker
-              const Mk q = TV.next_beyond(C, side, k, j);
-              if (q.kind >= 0) {
-                const uint16_t qr = TV.ref(q);
-                third(qr, TV.own_fraction(qr));
-              } else {
-                use = false;
-              }
-            }
-            if (use) ok = circle_cross_r(ay, x0, cx, cy, c2, rx, ry, r2, tfar, &ys);
+      const bool want = act && !online && !line_only && !d_below_sep(c2) && (C.fl & (side ? CF_P4 : CF_P1));
+      const unsigned wanted = __ballot_sync(kFull, want);
+      if (want) {
+        double X, Y, rx, ry, r2;
+        bool tfar, use = true;
+        if constexpr (sizeof(R) == 4) {
+          // its offsets from A exactly; its distance from B only where a float
+          // estimate (error below 2e-6 per component) does not already put it
+          // clearly past the minimum separation
+          float Xf, Yf;
+          TV.xyf(side ? C.p4 : C.p1, k, j, fy_t, &X, &Y, &Xf, &Yf);
+          rx = X - ax;
+          ry = Y - ay;
+          r2 = rx * rx + ry * ry;
+          const float txf = Xf - bxf, tyf = Yf - byf;
+          if (txf * txf + tyf * tyf >= 1.5e-4f) {
+            tfar = true;
           } else {
-            double X, Y;
-            TV.xy(side ? C.p4 : C.p1, k, j, &X, &Y);
-            FitPt T = fit_pt(X, Y, ax, ay, bx, by);
-            bool use = true;
-            if (d_below_sep(side ? T.t2 : T.r2)) {  // too close to A (B): the next marker
-              const Mk q = TV.next_beyond(C, side, k, j);
-              if (q.kind >= 0) {
-                TV.xy(TV.ref(q), k, j, &X, &Y);
-                T = fit_pt(X, Y, ax, ay, bx, by);
-              } else {
-                use = false;
-              }
-            }
-            if (use) ok = circle_cross(ay, x0, cx, cy, c2, T, &ys);
+            const double tx = X - bx, ty = Y - by;
+            tfar = !d_below_sep(tx * tx + ty * ty);
           }
+        } else {
+          TV.xy(side ? C.p4 : C.p1, k, j, &X, &Y);
+          const FitPt third = fit_pt(X, Y, ax, ay, bx, by);
+          rx = third.rx;
+          ry = third.ry;
+          r2 = third.r2;
+          tfar = !d_below_sep(third.t2);
         }
+        if (side ? !tfar : d_below_sep(r2)) {  // too close to B (A): the next marker
+          const NextPt q = next_point(TV, item >> 1, side, k, j, ax, ay, bx, by);
+          use = q.found;
+          rx = q.T.rx;
+          ry = q.T.ry;
+          r2 = q.T.r2;
+          tfar = !d_below_sep(q.T.t2);
+        }
+        __syncwarp(wanted);
+        if (use) ok = circle_cross_r(ay, x0, cx, cy, c2, rx, ry, r2, tfar, &ys);
       }
       const double yo = __shfl_xor_sync(kFull, ys, 1);
       const bool oko = __shfl_xor_sync(kFull, (int)ok, 1) != 0;
@@ -878,7 +1039,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
           y = by;
           kind = D_FIT_ONLINE;
         } else if (ok && oko) {
-          y = 0.5 * (ys + yo);
+          y = d_scale<-1>(ys + yo);
           kind = D_FIT_TWO;
         } else if (ok || oko) {
           y = ok ? ys : yo;
@@ -888,7 +1049,6 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
           kind = D_FIT_LINE;
         }
         C.y = y;
-        if (sizeof(R) == 4) C.sf = to_fraction<float>(y);  // here, where the FP64 pipe is busy anyway
         C.kind = (int8_t)kind;
         if (C.fl & CF_OWNED) {  // static indices keep the counters in registers
 #pragma unroll
@@ -904,7 +1064,8 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
     const int ne = s_ne;
     n_canc = 0;
     n_inv = 0;
-    for (int w = tid; w < ne && tid < kSplit; w += kSplit) {
+#pragma unroll 1
+    for (int w = tid; w < ne; w += kTileThreads) {
       const int id = M.u.c.le[w], ex = id % kRX, ey = id / kRX;
       if (getb(M.ovf, ex, ey)) continue;
       const int k = ri0 + ex, j = rj0 + ey;
@@ -912,8 +1073,18 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       const bool own = k < i0 + kTI;
       const int present = getb(M.kn, ex, ey) ^ getb(M.kn, ex, ey + 1);
       const uint32_t hd = (M.head[e / kHPW] >> ((e % kHPW) * kHB)) & kHNone;
-      int kept;
-      const NewV<R> nv = select_linked<R>(M, hd == kHNone ? -1 : (int)hd, present, &kept);
+      int kept = -1;
+      NewV<R> nv;
+      if (hd != kHNone && M.u.c.next[hd] < 0 && present) {
+        // one candidate on an edge that keeps a marker: it is the marker
+        kept = (int)hd;
+        nv.present = 1;
+        nv.cancelled = 0;
+        nv.invariant = 0;
+        nv.s = to_fraction<R>(M.u.c.cand[hd].y);
+      } else {
+        nv = select_rare<R, CAP>(M, hd == kHNone ? -1 : (int)hd, present, &kept);
+      }
       if (own) {
         n_canc += nv.cancelled;
         n_inv += nv.invariant;
@@ -921,28 +1092,14 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       // centre-rule verdicts of the kept candidate (Sec. 2.3), for the cells
       // either side of the edge that have four markers after the sweep (the
       // only ones whose centre colour the rule sets)
-      int vr = -1, vl = -1;
       if (kept >= 0) {
         auto four = [&](int x) {  // cell (x, ey) of the region, new colours
-          const int a = getb(M.kn, x, ey), b = getb(M.kn, x + 1, ey);
-          const int c = getb(M.kn, x + 1, ey + 1), d = getb(M.kn, x, ey + 1);
-          return a != b && b != c && c != d;
+          const int q = corners4(M.kn, x, ey);
+          return q == 5 || q == 10;
         };
         const bool fr = four(ex), fl = four(ex - 1);
-        if (fr || fl) {
-          const Cand& C = M.u.c.cand[kept];
-          const Mk none{-1, 0, 0};
-          if (fr) {
-            const int lr = walk(TV, TV.mk(C.b), (C.fl & CF_P4) ? TV.mk(C.p4) : none, k);
-            vr = lr < 0 ? -1 : !TV.knew(k, lr);
-          }
-          if (fl) {
-            const int ll = walk(TV, TV.mk(C.a), (C.fl & CF_P1) ? TV.mk(C.p1) : none, k - 1);
-            vl = ll < 0 ? -1 : !TV.knew(k, ll);
-          }
-        }
+        if (fr || fl) M.vrl[e] = verdicts_of(TV, kept, k, fr, fl);
       }
-      M.vrl[e] = verdicts(vr, vl);
       if (own && nv.present) {
         if (AX) { if (in_range((long long)k * P + j, G.d.nH())) out.sH[(long long)k * P + j] = nv.s; }
         else if (in_range((long long)j * P + k, G.d.nV())) out.sV[(long long)j * P + k] = nv.s;
@@ -955,7 +1112,8 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       // fraction 0.5
       uint32_t miss = (M.kn[u] ^ M.kn[u + kRW]) & ~M.hc[u] & ~M.ovf[u] &
                       span_mask(wi, max(4, 1 - ri0), min(kTI + 3, tnx - 1 - ri0));
-      while (miss) {
+  #pragma unroll 1
+    while (miss) {
         const int b = __ffs(miss) - 1;
         miss &= miss - 1;
         const int k = ri0 + 32 * wi + b, j = rj0 + ly;
@@ -967,8 +1125,10 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
     // edges whose candidates did not fit in the tile's list are done in
     // place by the generic logic, spread over all threads: overflow edge m
     // (in word order) goes to thread m mod the block size
+#pragma unroll 1
     for (int m = tid; m < s_novf; m += kTileThreads) {
       int u = 2 * kRW, r = m;
+#pragma unroll 1
       for (; u < kRB; ++u) {
         const int c = __popc(M.ovf[u]);
         if (r < c) break;
@@ -976,6 +1136,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       }
       if (u >= kRB) break;  // not reached: s_novf counts these words' bits
       uint32_t o = M.ovf[u];
+#pragma unroll 1
       for (; r > 0; --r) o &= o - 1;
       const int b = __ffs(o) - 1, ly = u / kRW, wi = u % kRW;
       const int k = ri0 + 32 * wi + b, j = rj0 + ly;
@@ -984,7 +1145,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       int oc[D_NUSED];
 #pragma unroll
       for (int c = 0; c < D_NUSED; ++c) oc[c] = 0;
-      const NewV<R> nv = new_unaligned<R>(TV, line_only != 0, k, j, own ? oc : nullptr);
+      const NewV<R> nv = new_unaligned_rare<R>(TV, line_only != 0, k, j, own ? oc : nullptr);
       for (int c = 0; c < D_NUSED; ++c)
         if (oc[c]) atomicAdd(&s_cnt[c], oc[c]);
       M.vrl[e] = verdicts(nv.vr, nv.vl);
@@ -1015,6 +1176,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       const uint32_t a1 = bits32(M.kn, ly, cx0 + 1);
       const uint32_t b0 = bits32(M.kn, ly + 1, cx0), b1 = bits32(M.kn, ly + 1, cx0 + 1);
       uint32_t fm = (kw ^ a1) & (b0 ^ b1) & (kw ^ b0) & cmask;
+#pragma unroll 1
       while (fm) {
         const int b = __ffs(fm) - 1;
         fm &= fm - 1;
@@ -1063,11 +1225,11 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
 }
 
 // One grid: block (bx, by) runs the tile at (64 bx, 32 by).
-template <typename R, int AX>
-__global__ void __launch_bounds__(tile_threads<R>(), tile_min_blocks<R>())
+template <typename R, int AX, int T>
+__global__ void __launch_bounds__(T, T == tile_threads<R>() ? tile_min_blocks<R>() : 4)
 k_sweep_tile(GView<R, AX> G, Buf<R> out, int line_only, unsigned long long* ctr,
              unsigned long long* cfl_bits, int* status) {
-  sweep_tile<R, AX>(G, out, line_only, ctr, cfl_bits, status, blockIdx.x * kTI, blockIdx.y * kTJ);
+  sweep_tile<R, AX, 0, kCandCap, T>(G, out, line_only, ctr, cfl_bits, status, blockIdx.x * kTI, blockIdx.y * kTJ);
 }
 
 // Many grids in one launch: per-grid sweep descriptors and a list of work
