@@ -5,12 +5,15 @@
 // stencils.
 //
 // Colours are read as bit rows; full, empty and interface cells are word
-// operations on them.  FP64 work is confined to interface cells: a full or
-// empty cell has C equal to its corner colour exactly, so full cells are
-// counted as integers and only interface fractions enter the double partial
-// sums.  The interface cells are listed in region order (a deterministic scan)
-// and each thread sums its list entries in order, then fixed shuffle and block
-// orders, which keeps the sums deterministic.
+// operations on them.  A full or empty cell has C equal to its corner colour
+// exactly: C and a NaN kappa are stored four cells at a time from the words,
+// and the interface cells, listed in region order, overwrite theirs.  FP64
+// work is confined to them, and there to what has to be double: the area is
+// added up as integers (exactly, in any order) and so are the heights of the
+// double form.  What bounds it then is instruction issue and the dense stores:
+// 4096^2 cells with 1.2 M interface cells, 118 -> 88 us in FP32 and 322 -> 140
+// us in FP64 (with double heights and sums the FP64 pipe was busy 82% of the
+// time); 2.2 and 2.9 TB/s of the dense model, state read and C, kappa written.
 #pragma once
 #include "ebit_device.cuh"
 
@@ -20,54 +23,45 @@ constexpr int kFX = 64, kFY = 32, kFH = 3;
 constexpr int kFRX = kFX + 2 * kFH, kFRY = kFY + 2 * kFH;  // region cells (70 x 38)
 constexpr int kFVX = kFRX + 1, kFVY = kFRY + 1;            // region vertices (71 x 39)
 constexpr int kFW = 3;                                     // words per region bit row
-// Threads per tile and blocks per SM the kernel is compiled for: eight float
-// tiles of 256 threads (32 registers, a few spilled, 12% faster than the five
-// that 48 registers allow; 384 or 512 threads per tile were slower); the
-// double form's shared memory admits seven at most, and it gains nothing.
+constexpr int kFP = 72;  // row pitch of the region's fractions: cell lx is entry lx + 1, so that
+                         // groups of four entries are groups of four of the tile's columns
+// Threads per tile and blocks per SM the kernel is compiled for: 4096^2 cells
+// take 88 us in FP32 with eight blocks of 32 registers (a few spilled), 99 with
+// six, 111 with five; in FP64 140 us with six, 143 with five, 171 with seven.
 template <typename R> __host__ __device__ constexpr int field_threads() { return 256; }
-template <typename R> __host__ __device__ constexpr int fields_min_blocks() { return sizeof(R) == 4 ? 8 : 5; }
+template <typename R> __host__ __device__ constexpr int fields_min_blocks() { return sizeof(R) == 4 ? 8 : 6; }
 
-// Reference-phase area of cell (i,j) in cell units from its corner mask q,
-// centre colour and marker fractions; double arithmetic.  The one-minus
-// terms are formed once and each case then takes a few operations, so that a
-// warp whose cells fall in different cases repeats little FP64 work.
+// Reference-phase area of interface cell (i,j) in cell units from its corner
+// mask q, centre colour and marker fractions; double arithmetic.  Two markers
+// on edges e1 < e2 cut a corner off (legs a and b) or leave a trapezoid (sides
+// a and b), each the marker's fraction or its one-minus: one sequence for all
+// of them, so that a warp whose cells differ repeats no FP64 work.
 template <typename R>
-__device__ double fraction_of(int q, int zc, const R* __restrict__ sH, const R* __restrict__ sV,
-                              const Dims& d, int i, int j) {
-  const int em = edge_mask(q);
+__device__ __forceinline__ double fraction_of(int q, int zc, const R* __restrict__ sH, const R* __restrict__ sV,
+                                              const Dims& d, int i, int j) {
+  const long long q0 = (long long)j * d.P + i;
   // exact conversions on the integer pipe
-  const long long q0 = (long long)j * d.P + i, q2 = q0 + d.P;  // sH of edges 0, 2; sV of 3, 1 at q0, q0 + 1
-  const double s0 = in_range(q0, d.nH()) ? to_d<R>(__ldg(&sH[q0])) : 0.0;
-  const double s1 = in_range(q0 + 1, d.nV()) ? to_d<R>(__ldg(&sV[q0 + 1])) : 0.0;
-  const double s2 = in_range(q2, d.nH()) ? to_d<R>(__ldg(&sH[q2])) : 0.0;
-  const double s3 = in_range(q0, d.nV()) ? to_d<R>(__ldg(&sV[q0])) : 0.0;
-  // legs of the triangle cut off at corner c: (s3, s0) (1-s0, s1) (1-s1, 1-s2)
-  // (s2, 1-s3); a one-minus is formed only for the legs that take it
-  auto tri = [&](int c) {
-    const double xa = c == 0 ? s3 : c == 1 ? s0 : c == 2 ? s1 : s2;
-    const double xb = c == 0 ? s0 : c == 1 ? s1 : c == 2 ? s2 : s3;
-    const double a = (c == 1 || c == 2) ? 1.0 - xa : xa;
-    const double b = (c >= 2) ? 1.0 - xb : xb;
-    return 0.5 * (a * b);
+  auto marker = [&](int e) {
+    const long long at = e == 1 ? q0 + 1 : e == 2 ? q0 + d.P : q0;
+    return in_range(at, e & 1 ? d.nV() : d.nH()) ? to_d<R>(__ldg(e & 1 ? &sV[at] : &sH[at])) : 0.0;
   };
+  const int em = edge_mask(q);
   if (em != 15) {
     const int e1 = __ffs(em) - 1, e2 = 31 - __clz(em);
-    const int c0 = q & 1;
-    if (e2 - e1 == 2) {  // opposite edges: a trapezoid
-      const double xa = e1 == 0 ? s0 : s3;
-      const double xb = e1 == 0 ? s2 : s1;
-      const double a = c0 ? xa : 1.0 - xa;
-      const double b = c0 ? xb : 1.0 - xb;
-      return 0.5 * (a + b);
-    }
-    const int c = (e1 == 0 && e2 == 3) ? 0 : e2;
-    const double T = tri(c);
-    return ((q >> c) & 1) ? T : 1.0 - T;
+    double a = marker(e1), b = marker(e2);
+    const bool opposite = e2 - e1 == 2;
+    const int c = e2 - e1 == 3 ? 0 : e2;  // the corner cut off
+    if (opposite ? !(q & 1) : (c == 1 || c == 2)) a = 1.0 - a;
+    if (opposite ? !(q & 1) : c >= 2) b = 1.0 - b;
+    double f = d_scale<-1>(opposite ? a + b : a * b);
+    if (!opposite && !((q >> c) & 1)) f = 1.0 - f;
+    return f;
   }
   // four markers: the two corners of the other colour than the centre are cut
   // off (corners 1 and 3 when corner 0 has the centre's colour, else 0 and 2)
-  const int ca = ((q & 1) == zc) ? 1 : 0;
-  const double Tsum = tri(ca) + tri(ca + 2);
+  const double s0 = marker(0), s1 = marker(1), s2 = marker(2), s3 = marker(3);
+  const double Tsum = (q & 1) == zc ? 0.5 * ((1.0 - s0) * s1) + 0.5 * (s2 * (1.0 - s3))
+                                    : 0.5 * (s3 * s0) + 0.5 * ((1.0 - s1) * (1.0 - s2));
   return zc == 0 ? Tsum : 1.0 - Tsum;
 }
 
@@ -79,14 +73,118 @@ __device__ __forceinline__ uint32_t fshr1(const uint32_t* w, int ly, int wi) {
   if (wi + 1 < kFW) v |= w[ly * kFW + wi + 1] << 31;
   return v;
 }
+// Corner mask of region cell (lx, ly); kw has a word after its last row.
+__device__ __forceinline__ int fcorners(const uint32_t* kw, int lx, int ly) {
+  const uint32_t* q = kw + ly * kFW + (lx >> 5);
+  const int lo = __funnelshift_r(q[0], q[1], lx & 31) & 3;
+  const int up = __funnelshift_r(q[kFW], q[kFW + 1], lx & 31) & 3;
+  return lo | ((up & 2) << 1) | ((up & 1) << 3);
+}
 
-// Dense stores of four consecutive values of a row (16-byte aligned for float).
+// A fraction 0 <= f <= 1 in units of 2^-60, rounded down; a positive one is at
+// least one unit, so that only 0 is 0 and only 1 is 2^60.
+typedef unsigned long long fix60;
+constexpr fix60 kFixOne = 1ull << 60;
+__device__ __forceinline__ fix60 to_fix60(double f) {
+  const unsigned long long u = (unsigned long long)dbits(f) & 0x7fffffffffffffffull;
+  const int sh = 1015 - (int)(u >> 52);  // f = sig 2^(8 - sh) units
+  const unsigned long long sig = significand(u);
+  if (u == 0) return 0;
+  if (sh <= 0) return sig << -sh;
+  return sh > 52 ? 1ull : sig >> sh;
+}
+// (double)v 2^-60 for |v| < 2^63, to 53 bits (rounded toward zero).
+__device__ __forceinline__ double from_fix60(long long v) {
+  if (v == 0) return 0.0;
+  const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int p = 63 - __clzll((long long)a);
+  const unsigned long long sig = p > 52 ? a >> (p - 52) : a << (52 - p);
+  return __longlong_as_double((long long)((v < 0 ? 1ull << 63 : 0ull) |
+                                          ((unsigned long long)(1023 + p - 60) << 52) | (sig & (kImplicit - 1))));
+}
+
+// What the height functions add up.  The float form adds floats in stencil
+// order, as the definition spells it.  The double form adds integers in units
+// of 2^-60: exact sums, finer than the double fractions they are made of
+// (2^-54 for those above a half), and none of the 21 additions of a stencil
+// takes a slot of the FP64 pipe.
+template <typename R> struct HeightOf;
+template <> struct HeightOf<float> {
+  typedef float T;
+  static __device__ __forceinline__ float one() { return 1.0f; }
+  static __device__ __forceinline__ float of(double, float f) { return f; }
+};
+template <> struct HeightOf<double> {
+  typedef fix60 T;
+  static __device__ __forceinline__ fix60 one() { return kFixOne; }
+  static __device__ __forceinline__ fix60 of(double f, double) { return to_fix60(f); }
+};
+__device__ __forceinline__ bool is_one(float h) { return one_bits(h); }
+__device__ __forceinline__ bool is_one(fix60 h) { return h == kFixOne; }
+__device__ __forceinline__ bool is_zero(float h) { return zero_bits(h); }
+__device__ __forceinline__ bool is_zero(fix60 h) { return h == 0; }
+
+// kappa from the heights of the three columns.
+__device__ __forceinline__ float height_kappa(const float h[3], float dx) {
+  const float hp = (h[2] - h[0]) * 0.5f;
+  const float hpp = (h[2] - h[1]) - (h[1] - h[0]);
+  const float qv = 1.0f + hp * hp;
+  const float den = dx * (qv * sqrt(qv));
+  return -hpp / den;
+}
+__device__ __forceinline__ double height_kappa(const fix60 h[3], double dx) {
+  const double hp = d_scale<-1>(from_fix60((long long)(h[2] - h[0])));
+  const double hpp = from_fix60((long long)((h[2] - h[1]) - (h[1] - h[0])));
+  const double qv = 1.0 + hp * hp;
+  const double den = dx * (qv * d_sqrt(qv));
+  return -d_div(hpp, den);
+}
+
+// Heights run along y when the segments' |dx| add up to at least their |dy|.
+template <typename R>
+__device__ __forceinline__ bool along_y(int ns, const int seg[2][2], const R px[4], const R py[4], R* margin) {
+  R ax = R(0), ay = R(0);
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    if (s >= ns) break;
+    ax = ax + fabs(px[seg[s][1]] - px[seg[s][0]]);
+    ay = ay + fabs(py[seg[s][1]] - py[seg[s][0]]);
+  }
+  *margin = fabs(ax - ay);
+  return ax >= ay;
+}
+__device__ __forceinline__ bool heights_along_y(int ns, const int seg[2][2], const float px[4], const float py[4]) {
+  float m;
+  return along_y(ns, seg, px, py, &m);
+}
+// The double form decides on float estimates (each coordinate within 2^-20, so
+// the sums' difference within 2^-17) and takes the FP64 pipe only where they
+// are too close to tell.
+__device__ __forceinline__ bool heights_along_y(int ns, const int seg[2][2], const double px[4],
+                                                const double py[4]) {
+  float fx[4], fy[4], m;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    fx[e] = d_mid(px[e]) ? d_top(px[e]) : 0.0f;
+    fy[e] = d_mid(py[e]) ? d_top(py[e]) : 0.0f;
+  }
+  const bool y = along_y(ns, seg, fx, fy, &m);
+  if (m > 0x1p-16f) return y;
+  double md;
+  return along_y(ns, seg, px, py, &md);
+}
+
+// Dense stores of four consecutive values of a row (16-byte aligned).
 __device__ __forceinline__ void store4(float* p, float a, float b, float c, float d) {
   *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
 }
 __device__ __forceinline__ void store4(double* p, double a, double b, double c, double d) {
   reinterpret_cast<double2*>(p)[0] = make_double2(a, b);
   reinterpret_cast<double2*>(p)[1] = make_double2(c, d);
+}
+__device__ __forceinline__ void store4(fix60* p, fix60 a, fix60 b, fix60 c, fix60 d) {
+  reinterpret_cast<ulonglong2*>(p)[0] = make_ulonglong2(a, b);
+  reinterpret_cast<ulonglong2*>(p)[1] = make_ulonglong2(c, d);
 }
 
 // Where the tiles' area partials are summed: with `done` set, the last tile
@@ -114,24 +212,24 @@ __device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
                                             int* ghf_list = nullptr, unsigned* ghf_count = nullptr,
                                             AreaSum sum = AreaSum()) {
   constexpr int kFieldThreads = field_threads<R>();
-  __shared__ uint32_t kw[kFVY * kFW];  // vertex colours
+  typedef HeightOf<R> H;
+  typedef typename H::T HT;
+  __shared__ uint32_t kw[kFVY * kFW + 1];  // vertex colours
   __shared__ uint32_t zw[kFRY * kFW];  // centre colours
-  __shared__ uint32_t fw[kFRY * kFW];  // full cells
-  __shared__ uint32_t iw[kFRY * kFW];  // interface cells
-  __shared__ R cs[kFRY * kFRX];        // fractions of the region
-  __shared__ uint16_t lst[kFRY * kFRX];
-  __shared__ int s_woff[kFieldThreads / 32];
-  __shared__ double s_wsum[kFieldThreads / 32];
+  __shared__ uint32_t fw[kFRY * kFW + 1];  // full cells
+  __shared__ uint32_t iw[kFRY * kFW];      // interface cells
+  __shared__ __align__(16) HT cs[kFRY * kFP];  // fractions of the region
+  __shared__ uint16_t lst[kFRY * kFRX];        // interface cells, in region order (entries of cs)
   __shared__ int s_cnt[D_NUSED];
-  __shared__ unsigned long long s_full;
+  __shared__ unsigned long long s_area;  // the tile's area, units of 2^-52 cells
   __shared__ unsigned s_nghf, s_ghf_base;
-  __shared__ int s_last;
+  __shared__ int s_last, s_n;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int i0 = bx * kFX, j0 = by * kFY;
   const int rx0 = i0 - kFH, ry0 = j0 - kFH;
   if (tid < D_NUSED) s_cnt[tid] = 0;
   if (tid == 0) {
-    s_full = 0ull;
+    s_area = 0ull;
     s_nghf = 0u;
   }
   // region columns / rows inside the grid
@@ -139,9 +237,7 @@ __device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
   const int cx1 = min(kFRX - 1, d.nx - 1 - rx0);                  // cells
   const int vy0 = max(0, -ry0), vy1 = min(kFVY - 1, d.ny - ry0);
   const int cy1 = min(kFRY - 1, d.ny - 1 - ry0);
-  int cnt[D_NUSED];
-#pragma unroll
-  for (int c = 0; c < D_NUSED; ++c) cnt[c] = 0;
+  int n_h = 0, n_v = 0, n_invalid = 0;
 
   // colour bits
   for (int t = tid; t < (kFVY + kFRY) * kFW; t += kFieldThreads) {
@@ -158,8 +254,9 @@ __device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
   __syncthreads();
 
   // full / interface cells; the tile's full cells and markers are counted
+  constexpr int kWords = kFRY * kFW;  // 114
   int full = 0;
-  for (int t = tid; t < kFRY * kFW; t += kFieldThreads) {
+  for (int t = tid; t < kWords; t += kFieldThreads) {
     const int ly = t / kFW, wi = t % kFW;
     uint32_t f = 0u, ic = 0u;
     if (ly >= vy0 && ly <= cy1) {
@@ -176,88 +273,101 @@ __device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
       // markers on the tile's vertices' right and upper edges
       if (ly <= vy1) {
         const uint32_t a = kw[t];
-        cnt[D_NH] += __popc((a ^ fshr1(kw, ly, wi)) & tile & span_mask(wi, vx0, cx1));
-        if (ly + 1 <= vy1) cnt[D_NV] += __popc((a ^ kw[t + kFW]) & tile & span_mask(wi, vx0, vx1));
+        n_h += __popc((a ^ fshr1(kw, ly, wi)) & tile & span_mask(wi, vx0, cx1));
+        if (ly + 1 <= vy1) n_v += __popc((a ^ kw[t + kFW]) & tile & span_mask(wi, vx0, vx1));
       }
     }
   }
   {
     const int fsum = __reduce_add_sync(0xffffffffu, full);
-    if (lane == 0 && fsum) atomicAdd(&s_full, (unsigned long long)fsum);
+    if (lane == 0 && fsum) atomicAdd(&s_area, (unsigned long long)fsum << 52);
   }
   __syncthreads();
 
-  // interface list in region order: per-warp scans of the word counts
-  constexpr int kWords = kFRY * kFW;  // 114
-  int pos = 0, n = 0;
-  uint32_t mybits = 0u;
-  if (warp < (kWords + 31) / 32) {
-    const int t = warp * 32 + lane;
-    mybits = t < kWords ? iw[t] : 0u;
-    n = __popc(mybits);
+  // interface list in region order: two words a lane of the first two warps,
+  // the cells before the second warp's words counted by itself
+  if (warp < 2) {
+    static_assert(kWords <= 128, "two words a lane, two warps");
+    const int t = 64 * warp + 2 * lane;
+    uint32_t w0 = t < kWords ? iw[t] : 0u, w1 = t + 1 < kWords ? iw[t + 1] : 0u;
+    const int n = __popc(w0) + __popc(w1);
+    const int before = warp ? __reduce_add_sync(0xffffffffu, __popc(iw[lane]) + __popc(iw[lane + 32])) : 0;
     int incl = n;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int v = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += v;
     }
-    pos = incl - n;
-    if (lane == 31) s_woff[warp] = incl;
+    int pos = before + incl - n;
+    if (warp == 1 && lane == 31) s_n = pos + n;
+    const int r0 = (t / kFW) * kFP + 32 * (t % kFW) + 1;
+    const int r1 = ((t + 1) / kFW) * kFP + 32 * ((t + 1) % kFW) + 1;
+    for (; w0; w0 &= w0 - 1) lst[pos++] = (uint16_t)(r0 + __ffs(w0) - 1);
+    for (; w1; w1 &= w1 - 1) lst[pos++] = (uint16_t)(r1 + __ffs(w1) - 1);
   }
-  // fractions of full and empty cells, a warp per region row
-  for (int ly = warp; ly < kFRY; ly += kFieldThreads / 32) {
-#pragma unroll
-    for (int w = 0; w < kFW; ++w) {
-      const int lx = 32 * w + lane;
-      const uint32_t f = fw[ly * kFW + w], ic = iw[ly * kFW + w];
-      if (lx < kFRX && !((ic >> lane) & 1u)) cs[ly * kFRX + lx] = ((f >> lane) & 1u) ? R(1) : R(0);
+  // Full and empty cells, four at a time: the region's for the heights, and
+  // the tile's straight to C, with NaN to kappa (the interface cells' entries
+  // are written after the next barriers).
+  {
+    const bool vec = ((reinterpret_cast<uintptr_t>(C) | reinterpret_cast<uintptr_t>(kappa)) & 15) == 0;
+    const HT one = H::one();
+    const R nan = R(NAN);
+    constexpr int kQ = kFP / 4;
+    for (int g = (tid + kFieldThreads - 64) % kFieldThreads; g < kFRY * kQ; g += kFieldThreads) {
+      const int ly = g / kQ, qx = g - ly * kQ, lx = 4 * qx - 1;  // its first cell (-1 for qx = 0)
+      const int w = ly * kFW + (lx >> 5);
+      const uint32_t f = qx == 0 ? fw[ly * kFW] << 1 : __funnelshift_r(fw[w], fw[w + 1], lx & 31);
+      store4(&cs[ly * kFP + 4 * qx], f & 1 ? one : HT(0), f & 2 ? one : HT(0), f & 4 ? one : HT(0),
+             f & 8 ? one : HT(0));
+      const int i = i0 + 4 * qx - 4, j = ry0 + ly;
+      if (qx == 0 || qx > kFX / 4 || ly < kFH || ly >= kFH + kFY || j >= d.ny || i >= d.nx) continue;
+      if (!in_range((long long)j * d.P + min(i + 3, d.nx - 1), d.nV())) continue;  // this group's last cell
+      R* Cp = C + (long long)j * d.P + i;
+      R* Kp = kappa + (long long)j * d.P + i;
+      const R c0 = f & 1 ? R(1) : R(0), c1 = f & 2 ? R(1) : R(0), c2 = f & 4 ? R(1) : R(0), c3 = f & 8 ? R(1) : R(0);
+      if (vec && i + 3 < d.nx) {
+        store4(Cp, c0, c1, c2, c3);
+        store4(Kp, nan, nan, nan, nan);
+      } else {
+        Cp[0] = c0;
+        Kp[0] = nan;
+        if (i + 1 < d.nx) { Cp[1] = c1; Kp[1] = nan; }
+        if (i + 2 < d.nx) { Cp[2] = c2; Kp[2] = nan; }
+        if (i + 3 < d.nx) { Cp[3] = c3; Kp[3] = nan; }
+      }
     }
   }
-  __syncthreads();
-  if (warp < (kWords + 31) / 32) {
-    for (int w = 0; w < warp; ++w) pos += s_woff[w];
-    const int t = warp * 32 + lane;
-    const int row0 = (t / kFW) * kFRX + 32 * (t % kFW);
-    while (mybits) {
-      const int b = __ffs(mybits) - 1;
-      mybits &= mybits - 1;
-      lst[pos++] = (uint16_t)(row0 + b);
-    }
-  }
-  int nlist = 0;
-#pragma unroll
-  for (int w = 0; w < (kWords + 31) / 32; ++w) nlist += s_woff[w];
   __syncthreads();
 
-  // interface fractions (FP64 on full warps) and the tile's area
-  double acc = 0.0;
+  // interface fractions (FP64 on full warps) and the tile's area, added up as
+  // integers: exactly, whatever the order
+  const int nlist = s_n;
+  fix60 acc = 0;  // at most 11 cells a thread: below 2^64
+  static_assert((kFRY * kFRX + kFieldThreads - 1) / kFieldThreads <= 15, "a thread's area fits");
   for (int e = tid; e < nlist; e += kFieldThreads) {
-    const int t = lst[e];
-    const int lx = t % kFRX, ly = t / kFRX;
-    const int q = fgetb(kw, lx, ly) | (fgetb(kw, lx + 1, ly) << 1) |
-                  (fgetb(kw, lx + 1, ly + 1) << 2) | (fgetb(kw, lx, ly + 1) << 3);
-    const double f = fraction_of(q, fgetb(zw, lx, ly), sH, sV, d, rx0 + lx, ry0 + ly);
-    cs[t] = (R)f;
-    if (lx >= kFH && lx < kFH + kFX && ly >= kFH && ly < kFH + kFY) acc = acc + f;
+    const int t = lst[e], ly = t / kFP, lx = t - ly * kFP - 1;
+    const int i = rx0 + lx, j = ry0 + ly;
+    const double f = fraction_of(fcorners(kw, lx, ly), fgetb(zw, lx, ly), sH, sV, d, i, j);
+    const R c = (R)f;
+    cs[t] = H::of(f, c);
+    if (lx >= kFH && lx < kFH + kFX && ly >= kFH && ly < kFH + kFY) {
+      acc += to_fix60(f);
+      if (in_range((long long)j * d.P + i, d.nV())) C[(long long)j * d.P + i] = c;
+    }
   }
-  // area partial: warps holding interface cells reduce in a fixed shuffle
-  // order (adding 0.0 from the other lanes changes nothing)
-  if (__any_sync(0xffffffffu, !d_eq0(acc))) {
-    for (int o = 16; o > 0; o >>= 1) acc = acc + __shfl_down_sync(0xffffffffu, acc, o);
-  } else {
-    acc = 0.0;
+  if (__any_sync(0xffffffffu, acc != 0)) {
+    const unsigned long long a = (acc + 128) >> 8;  // units of 2^-52, below 2^56
+    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)a & 0xffffffu);
+    const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(a >> 24) & 0xffffffu);
+    const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(a >> 48));
+    if (lane == 0) atomicAdd(&s_area, lo + ((unsigned long long)mid << 24) + ((unsigned long long)hi << 48));
   }
-  if (lane == 0) s_wsum[warp] = acc;
   __syncthreads();
   // the tile's partial, and its count towards the launch's last tile, by the
-  // last thread: it has no global stores in flight to fence, and it rarely
-  // has curvature work, so the fence and the counter's round trip overlap
-  // the other threads' curvature
+  // last thread: it rarely has curvature work, so the fence and the counter's
+  // round trip overlap the other threads' curvature
   if (tid == kFieldThreads - 1) {
-    double p = 0.0;
-    for (int w = 0; w < kFieldThreads / 32; ++w) p = p + s_wsum[w];
-    if (s_full) p = p + (double)s_full;
-    partial[slot] = p;
+    partial[slot] = __ull2double_rn(s_area) * 0x1p-52;
     s_last = 0;
     if (sum.done) {
       __threadfence();  // the partial is visible before the count says so
@@ -267,12 +377,10 @@ __device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
 
   // height-function curvature of the tile's interface cells
   for (int e = tid; e < nlist; e += kFieldThreads) {
-    const int ci = lst[e];
-    const int lx = ci % kFRX, ly = ci / kFRX;
+    const int ci = lst[e], ly = ci / kFP, lx = ci - ly * kFP - 1;
     if (lx < kFH || lx >= kFH + kFX || ly < kFH || ly >= kFH + kFY) continue;
     const int i = rx0 + lx, j = ry0 + ly;
-    const int q = fgetb(kw, lx, ly) | (fgetb(kw, lx + 1, ly) << 1) |
-                  (fgetb(kw, lx + 1, ly + 1) << 2) | (fgetb(kw, lx, ly + 1) << 3);
+    const int q = fcorners(kw, lx, ly);
     R out = R(NAN);
     int seg[2][2];
     const int ns = segments(q, edge_mask(q) == 15 ? fgetb(zw, lx, ly) : 0, seg);
@@ -281,42 +389,28 @@ __device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
                      in_range(q2, d.nH()) ? __ldg(&sH[q2]) : R(0), R(0)};
     const R py[4] = {R(0), in_range(q0 + 1, d.nV()) ? __ldg(&sV[q0 + 1]) : R(0), R(1),
                      in_range(q0, d.nV()) ? __ldg(&sV[q0]) : R(0)};
-    R ax = R(0), ay = R(0);
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      if (s >= ns) break;
-      const int a = seg[s][0], b = seg[s][1];
-      ax = ax + fabs(px[b] - px[a]);
-      ay = ay + fabs(py[b] - py[a]);
-    }
-    const bool ycol = ax >= ay;
-    const bool inside = ycol ? (i - 1 >= 0 && i + 1 <= d.nx - 1 && j - 3 >= 0 && j + 3 <= d.ny - 1)
-                             : (j - 1 >= 0 && j + 1 <= d.ny - 1 && i - 3 >= 0 && i + 3 <= d.nx - 1);
-    bool valid = inside;
-    R h[3];
-    if (inside) {
+    const bool ycol = heights_along_y(ns, seg, px, py);
+    bool valid = ycol ? (i - 1 >= 0 && i + 1 <= d.nx - 1 && j - 3 >= 0 && j + 3 <= d.ny - 1)
+                      : (j - 1 >= 0 && j + 1 <= d.ny - 1 && i - 3 >= 0 && i + 3 <= d.nx - 1);
+    if (valid) {
+      const int along = ycol ? kFP : 1, across = ycol ? 1 : kFP;
+      HT h[3];
       int orient[3];
 #pragma unroll
       for (int m = -1; m <= 1; ++m) {
-        R a = R(0);
+        const HT* c = &cs[ci + m * across - 3 * along];
+        const HT lo = c[0], hi = c[6 * along];
+        HT a = HT(0) + lo;
 #pragma unroll
-        for (int s = -3; s <= 3; ++s)
-          a = a + (ycol ? cs[(ly + s) * kFRX + lx + m] : cs[(ly + m) * kFRX + lx + s]);
-        h[m + 1] = a;
-        const R lo = ycol ? cs[(ly - 3) * kFRX + lx + m] : cs[(ly + m) * kFRX + lx - 3];
-        const R hi = ycol ? cs[(ly + 3) * kFRX + lx + m] : cs[(ly + m) * kFRX + lx + 3];
-        orient[m + 1] = (one_bits(lo) && zero_bits(hi)) ? 1 : (zero_bits(lo) && one_bits(hi)) ? -1 : 0;
+        for (int s = 1; s < 6; ++s) a = a + c[s * along];
+        h[m + 1] = a + hi;
+        orient[m + 1] = (is_one(lo) && is_zero(hi)) ? 1 : (is_zero(lo) && is_one(hi)) ? -1 : 0;
       }
       valid = orient[0] != 0 && orient[0] == orient[1] && orient[1] == orient[2];
+      if (valid) out = height_kappa(h, dx);
     }
-    if (valid) {
-      const R hp = (h[2] - h[0]) * R(0.5);
-      const R hpp = (h[2] - h[1]) - (h[1] - h[0]);
-      const R qv = R(1) + hp * hp;
-      const R den = dx * (qv * sqrt(qv));
-      out = -hpp / den;
-    } else {
-      cnt[D_HF_INVALID] += 1;
+    if (!valid) {
+      n_invalid += 1;
       if (ghf_list) {  // flag the entry for the generalised fallbacks
         lst[e] = (uint16_t)(ci | 0x8000);
         atomicAdd(&s_nghf, 1u);
@@ -324,37 +418,13 @@ __device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
     }
     if (in_range((long long)j * d.P + i, d.nV())) kappa[(long long)j * d.P + i] = out;
   }
-  // dense outputs: C everywhere, kappa = NaN away from the interface (the
-  // interface cells' kappa is written above)
-  const bool vec = ((reinterpret_cast<uintptr_t>(C) | reinterpret_cast<uintptr_t>(kappa)) & 15) == 0;
-  for (int g = tid; g < kFX * kFY / 4; g += kFieldThreads) {
-    const int lx0 = (g % (kFX / 4)) * 4, ly0 = g / (kFX / 4);
-    const int i = i0 + lx0, j = j0 + ly0;
-    if (j >= d.ny || i >= d.nx) continue;
-    const int lx = lx0 + kFH, ly = ly0 + kFH;
-    const R* c = &cs[ly * kFRX + lx];
-    const uint32_t ib = (iw[ly * kFW + (lx >> 5)] >> (lx & 31)) |
-                        ((lx & 31) > 28 ? iw[ly * kFW + (lx >> 5) + 1] << (32 - (lx & 31)) : 0u);
-    if (!in_range((long long)j * d.P + min(i + 3, d.nx - 1), d.nV())) continue;  // this group's last cell
-    R* Cp = C + (long long)j * d.P + i;
-    R* Kp = kappa + (long long)j * d.P + i;
-    if (vec && i + 3 < d.nx) {
-      store4(Cp, c[0], c[1], c[2], c[3]);
-      if (!(ib & 15u)) store4(Kp, R(NAN), R(NAN), R(NAN), R(NAN));
-      else
-        for (int m = 0; m < 4; ++m)
-          if (!((ib >> m) & 1u)) Kp[m] = R(NAN);
-    } else {
-      for (int m = 0; m < 4 && i + m < d.nx; ++m) {
-        Cp[m] = c[m];
-        if (!((ib >> m) & 1u)) Kp[m] = R(NAN);
-      }
-    }
-  }
   // the counters this kernel keeps (markers, cells without a height stencil)
-  for (const int c : {(int)D_NH, (int)D_NV, (int)D_HF_INVALID}) {
-    const int s = __reduce_add_sync(0xffffffffu, cnt[c]);
-    if (s != 0 && lane == 0) atomicAdd(&s_cnt[c], s);
+  {
+    const int h = __reduce_add_sync(0xffffffffu, n_h), v = __reduce_add_sync(0xffffffffu, n_v);
+    const int x = __reduce_add_sync(0xffffffffu, n_invalid);
+    if (lane == 0 && h) atomicAdd(&s_cnt[D_NH], h);
+    if (lane == 0 && v) atomicAdd(&s_cnt[D_NV], v);
+    if (lane == 0 && x) atomicAdd(&s_cnt[D_HF_INVALID], x);
   }
   __syncthreads();
   if (tid < D_NUSED && s_cnt[tid] != 0) atomicAdd(&ctr[tid], (unsigned long long)s_cnt[tid]);
@@ -371,7 +441,7 @@ __device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
         const int ci = lst[e];
         if (!(ci & 0x8000)) continue;
         const int t = ci & 0x7fff;
-        const int i = rx0 + t % kFRX, j = ry0 + t / kFRX;
+        const int i = rx0 + t % kFP - 1, j = ry0 + t / kFP;
         ghf_list[s_ghf_base + atomicAdd(&s_nghf, 1u)] = j * d.nx + i;
       }
     }
