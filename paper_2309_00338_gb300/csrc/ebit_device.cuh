@@ -413,24 +413,6 @@ template <typename R> __device__ __forceinline__ double to_d(R x);
 template <> __device__ __forceinline__ double to_d<float>(float x) { return f2d(x); }
 template <> __device__ __forceinline__ double to_d<double>(double x) { return x; }
 
-// (double)n + (double)f for an integer |n| <= 7 and a float 0 <= f < 1, the
-// value the FP64 addition gives.  When f >= 2^-26 the sum has at most 53
-// significant bits, so it is exact and is formed by integer operations;
-// smaller f take the FP64 addition.
-__device__ __forceinline__ double add_nf(int n, float f) {
-  const unsigned u = __float_as_uint(f);
-  if (u == 0u) return i2d(n);
-  const int e = (int)(u >> 23);
-  if (e < 101 || n < -7 || n > 7) return i2d(n) + f2d(f);
-  const int sh = 150 - e;  // f = m 2^-sh with 24 <= sh <= 49
-  const long long S = (long long)n * (1ll << sh) + (long long)((u & 0x7fffffu) | 0x800000u);
-  const unsigned long long sign = S < 0 ? (1ull << 63) : 0ull;
-  const unsigned long long a = S < 0 ? (unsigned long long)(-S) : (unsigned long long)S;
-  const int p = 63 - __clzll((long long)a);  // leading bit; p <= sh + 3 <= 52
-  const unsigned long long mant = (a << (52 - p)) & 0xfffffffffffffull;
-  return __longlong_as_double((long long)(sign | ((unsigned long long)(1023 + p - sh) << 52) | mant));
-}
-
 // ---------------------------------------------------------------------------
 // Correctly rounded double division and square root on the integer and FP32
 // pipes, for the circle fits: long division and longhand square root with
@@ -472,7 +454,7 @@ __device__ __forceinline__ bool mid_exponent(unsigned long long bits) {
 
 __device__ __forceinline__ double d_div(double n, double d) {
   const unsigned long long un = (unsigned long long)dbits(n), ud = (unsigned long long)dbits(d);
-  if (!mid_exponent(un) || !mid_exponent(ud)) return n / d;
+  if (__builtin_expect(!mid_exponent(un) || !mid_exponent(ud), 0)) return n / d;
   unsigned long long A = significand(un);
   const unsigned long long b = significand(ud);
   const int lt = A < b;
@@ -496,7 +478,7 @@ __device__ __forceinline__ double d_div(double n, double d) {
 
 __device__ __forceinline__ double d_sqrt(double x) {
   const unsigned long long ux = (unsigned long long)dbits(x);
-  if ((long long)ux < 0 || !mid_exponent(ux)) return sqrt(x);
+  if (__builtin_expect((long long)ux < 0 || !mid_exponent(ux), 0)) return sqrt(x);
   const unsigned ex = (unsigned)(ux >> 52);
   const int odd = (ex & 1u) == 0u;  // of the exponent ex - 1023
   const unsigned long long m = significand(ux), X = m << odd;  // [1, 4) in units of 2^-52
@@ -583,7 +565,7 @@ __device__ __forceinline__ bool circle_cross_r(double Ay, double x0, double qx, 
     const float sf = pf - rf;
     const bool sure = d_mid(qx) && d_mid(ya) && d_mid(qy) && d_mid(x0) &&
                       fabsf(sf) > 0x1p-16f * (fabsf(pf) + fabsf(rf));
-    if (!sure || (sf > 0.0f) == kpos) {
+    if (__builtin_expect(!sure || (sf > 0.0f) == kpos, 0)) {
       const double sa = qx * ya - qy * x0;
       if (kpos ? d_gt0(sa) : d_lt0(sa)) {
         const double yb = h / kap;

@@ -47,10 +47,14 @@ template <int CAP> __host__ __device__ constexpr int head_bits() { return CAP <=
 template <int CAP> __host__ __device__ constexpr uint32_t head_none() {
   return (1u << head_bits<CAP>()) - 1u;
 }
-constexpr uint16_t kKindV = 0x8000;    // marker reference: region index | kKindV if unaligned
-constexpr int kSecond = 0x4000;        // segment reference: region index of its cell | kSecond for the
-                                       // second one of a four-marker cell
-static_assert(kRN <= kSecond, "region indices leave the flag bits free");
+// A place of the region, (lx, ly), as 13 bits, taken apart without a division.
+__device__ __forceinline__ int pack_xy(int lx, int ly) { return ly << 7 | lx; }
+__device__ __forceinline__ int lx_of(int id) { return id & 127; }
+__device__ __forceinline__ int ly_of(int id) { return (id >> 7) & 63; }
+static_assert(kRX <= 128 && kRY <= 64, "places fit");
+constexpr uint16_t kKindV = 0x8000;    // marker reference: place | kKindV if unaligned
+constexpr int kSecond = 0x4000;        // segment reference: place of its cell | kSecond for the second
+                                       // one of a four-marker cell
 
 // Block shape: four warps per tile, seven tiles per SM in the FP32 form (72
 // registers) and six in the FP64 form (80).  What a tile waits for is latency
@@ -83,7 +87,7 @@ enum { CF_P1 = 1, CF_P4 = 4, CF_OWNED = 16 };
 struct Cand {
   double y;
   uint16_t a, b, p1, p4;
-  uint16_t edge;  // (j - j0) * (kTI + 1) + (k - i0)
+  uint16_t edge;  // pack_xy(k - i0, j - j0)
   uint8_t fl, ord;
   int8_t kind;
 };
@@ -210,7 +214,7 @@ __device__ __forceinline__ void flush_count(int* s_cnt, int c, int v, int lane) 
 __device__ __forceinline__ void push_bits_warp(uint32_t bits, int t, int flag, uint16_t* list,
                                                int* count, int lane) {
   int base = warp_alloc(__popc(bits), count, lane);
-  const int row0 = ((t / kRW) * kRX + 32 * (t % kRW)) | flag;
+  const int row0 = pack_xy(32 * (t % kRW), t / kRW) | flag;
 #pragma unroll 1
   while (bits) {
     const int b = __ffs(bits) - 1;
@@ -247,6 +251,15 @@ __device__ __forceinline__ uint32_t upto32(int c0, int last) {
 }
 
 
+// n + f + kShift for a grid line number n and a fraction f (see xy_shifted).
+constexpr int kShift = 12;
+__device__ __forceinline__ bool shifted_sum(int n, float f, double* s) {
+  const unsigned u = __float_as_uint(f), e = u >> 23;
+  const unsigned long long m = (unsigned long long)(u ? (u & 0x7fffffu) | 0x800000u : 0u) << ((e - 101u) & 31u);
+  *s = __longlong_as_double((1026ll << 52) + ((long long)(n + kShift - 8) << 49) + (long long)m);
+  return (unsigned)(n + 4) < 8u && (u == 0u || e >= 101u);
+}
+
 // Accessor of the tile for the shared sweep logic (beyond, walk,
 // new_unaligned).  Indices are clamped into the region; the kernel only asks
 // inside it.
@@ -268,12 +281,11 @@ struct TViewB {
   __device__ __forceinline__ int knew(int i, int j) const { return getb(m->kn, cx(i), cy(j)); }
   __device__ __forceinline__ int corners(int i, int j) const { return corners4(m->kb, cx(i), cy(j)); }
   __device__ __forceinline__ uint16_t ref(Mk mk) const {
-    return (uint16_t)((cy(mk.j) * kRX + cx(mk.i)) | (mk.kind ? kKindV : 0));
+    return (uint16_t)(pack_xy(cx(mk.i), cy(mk.j)) | (mk.kind ? kKindV : 0));
   }
   // The marker of a reference.
   __device__ __forceinline__ Mk mk(uint16_t r) const {
-    const int t = r & (kKindV - 1), ly = t / kRX;
-    return Mk{(r & kKindV) ? 1 : 0, ri0 + t - ly * kRX, rj0 + ly};
+    return Mk{(r & kKindV) ? 1 : 0, ri0 + lx_of(r), rj0 + ly_of(r)};
   }
   // The marker beyond point 1 (side 0) or point 4 (side 1) of candidate C on
   // the unaligned edge (k, j): points 1 and 4 are the markers beyond A and B
@@ -312,7 +324,7 @@ struct TViewB {
   }
   // Moved point of a referenced marker relative to vertex (k, j).
   __device__ __forceinline__ void xy(uint16_t r, int k, int j, double* X, double* Y) const {
-    const int t = r & (kKindV - 1), ly = t / kRX, lx = t - ly * kRX;
+    const int lx = lx_of(r), ly = ly_of(r);
     // the same values as (double)n + (double)f; the conversions run on the
     // integer pipe and an aligned marker's y needs no addition
     if (r & kKindV) {
@@ -327,31 +339,25 @@ struct TViewB {
   // state; 0 for an aligned marker.
   __device__ __forceinline__ R own_fraction(uint16_t r) const {
     if (!(r & kKindV)) return R(0);
-    const int t = r & (kKindV - 1), ly = t / kRX, lx = t - ly * kRX;
+    const int lx = lx_of(r), ly = ly_of(r);
     return g.v(ri0 + lx, rj0 + ly);
   }
-  // The point in the FP32 form, given its own fraction fy: the exact sums by
-  // integer operations where they are exact (add_nf), and a float estimate
-  // (Xf, Yf) within 2^-22 of each coordinate.
-  __device__ __forceinline__ void xyf(uint16_t r, int k, int j, float fy, double* X, double* Y,
-                                      float* Xf, float* Yf) const {
-    const int t = r & (kKindV - 1), ly = t / kRX, lx = t - ly * kRX;
-    const int ny = rj0 + ly - j;
-    int nx;
-    float fx;
-    if (r & kKindV) {
-      nx = ri0 + lx + get2(m->vq, lx, ly) - 1 - k;
-      fx = (float)m->fr[m->rank(1, lx, ly)];
-      *Y = add_nf(ny, fy);
-    } else {
-      nx = ri0 + lx + get2(m->hq, lx, ly) - 1 - k;
-      fx = (float)m->fr[m->rank(0, lx, ly)];
-      fy = 0.0f;
-      *Y = i2d(ny);
-    }
-    *X = add_nf(nx, fx);
+  // The point in the FP32 form, given its own fraction fy, relative to an
+  // origin kShift cells left of and below vertex (k, j): there the sums of a
+  // small grid line number and a fraction of at least 2^-26 are exact doubles
+  // in [8, 16), formed by one integer addition.  Differences of two such
+  // points are those of the points relative to (k, j).  False where a sum is
+  // not of that kind.  (Xf, Yf): float estimates relative to (k, j), within
+  // 2^-22.
+  __device__ __forceinline__ bool xy_shifted(uint16_t r, int k, int j, float fy, double* X, double* Y, float* Xf,
+                                             float* Yf) const {
+    const int lx = lx_of(r), ly = ly_of(r), kind = r >> 15;
+    const int nx = ri0 + lx + get2(kind ? m->vq : m->hq, lx, ly) - 1 - k, ny = rj0 + ly - j;
+    const float fx = (float)m->fr[m->rank(kind, lx, ly)];
     *Xf = (float)nx + fx;
     *Yf = (float)ny + fy;
+    const bool ok = shifted_sum(nx, fx, X);
+    return shifted_sum(ny, fy, Y) && ok;
   }
 };
 
@@ -452,6 +458,12 @@ __device__ __noinline__ Landing<R> landing_rare(bool v0, bool v1, bool v2, R f0,
 template <typename R, int CAP>
 __device__ __noinline__ NewV<R> select_rare(const TileMem<R, CAP>& M, int s, int present, int* kept) {
   return select_linked<R>(M, s, present, kept);
+}
+
+// A referenced marker's moved point relative to vertex (k, j), out of line.
+template <typename R, int AX, int LD, int CAP>
+__device__ __noinline__ void xy_rare(const TViewB<R, AX, LD, CAP> TV, uint16_t r, int k, int j, double* X, double* Y) {
+  TV.xy(r, k, j, X, Y);
 }
 
 // The marker beyond point 1 (side 0) or 4 (side 1) of a candidate, as a third
@@ -720,8 +732,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       if (t0 < kRB) base[t0] = (uint16_t)at;
       if (t0 + 1 < kRB) base[t0 + 1] = (uint16_t)(at + n0);
       if (hf && lane == 31) (pl ? s_nm : s_nh) = at + n;
-      const int r0 = (t0 / kRW) * kRX + 32 * (t0 % kRW);
-      const int r1 = ((t0 + 1) / kRW) * kRX + 32 * ((t0 + 1) % kRW);
+      const int r0 = pack_xy(32 * (t0 % kRW), t0 / kRW), r1 = pack_xy(32 * ((t0 + 1) % kRW), (t0 + 1) / kRW);
 #pragma unroll 1
       for (; w0 && at < kMkCap; w0 &= w0 - 1) M.u.mk[at++] = (uint16_t)(r0 + __ffs(w0) - 1);
 #pragma unroll 1
@@ -743,7 +754,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
     R dmax = R(0);
 #pragma unroll 1
     for (int w = tid; w < nm; w += kTileThreads) {
-      const int id = M.u.mk[w], lx = id % kRX, ly = id / kRX;
+      const int id = M.u.mk[w], lx = lx_of(id), ly = ly_of(id);
       const int x = ri0 + lx, y = rj0 + ly;
       const bool al = w < nh;
       Flags f;
@@ -786,7 +797,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
     static_assert(kSplit > 0 && kSplit % 32 == 0, "warp split");
 #pragma unroll 1
     for (int w = tid; w < nh; w += kTileThreads) {
-      const int id = M.u.mk[w], lx = id % kRX, ly = id / kRX;
+      const int id = M.u.mk[w], lx = lx_of(id), ly = ly_of(id);
       const int dl = lx + get2(M.hq, lx, ly) - 1;
       if (dl < 1 || dl > kRX - 3) continue;
       const int x = ri0 + dl, y = rj0 + ly;
@@ -801,7 +812,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       if (lx != dl - 1 && (valid[0] || (lx != dl && valid[1]))) continue;  // a lower source's edge
       const int present = getb(M.kn, dl, ly) ^ getb(M.kn, dl + 1, ly);
       Landing<R> L;
-      if (present && (int)valid[0] + (int)valid[1] + (int)valid[2] == 1) {  // it stays
+      if (__builtin_expect(present && (int)valid[0] + (int)valid[1] + (int)valid[2] == 1, 1)) {  // it stays
         L = Landing<R>{1, ri0 + lx, 0, 0, M.fr[w]};
       } else {
         L = landing_rare<R>(valid[0], valid[1], valid[2], fx[0], fx[1], fx[2], x, present);
@@ -858,17 +869,16 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
     for (int w0 = warp * 32; w0 < nc; w0 += kTileThreads) {
       const int w = w0 + lane;
       int lx = 0, ly = 0, second = 0, ea = 0, eb = 0, xa = 0, klo = 0, khi = -1;
-      // edge e of the cell as a region index
-      auto at = [&](int e) { return (ly + (e == 2)) * kRX + lx + (e == 1); };
+      auto at = [&](int e) { return pack_xy(lx + (e == 1), ly + (e == 2)); };  // edge e of the cell
       if (w < nc) {
-        const int id = M.cl[w], cell = id & (kSecond - 1);
+        const int id = M.cl[w];
         second = id >= kSecond;
-        ly = cell / kRX;
-        lx = cell - ly * kRX;
+        ly = ly_of(id);
+        lx = lx_of(id);
         const int q = corners4(M.kb, lx, ly), em = edge_mask(q);
         ea = __ffs(em) - 1;
         eb = 31 - __clz(em);
-        if (em == 15) {  // the pairs of segments()
+        if (__builtin_expect(em == 15, 0)) {  // the pairs of segments()
           const bool same = (q & 1) == getb(M.zb, lx, ly);
           ea = same ? 2 * second : 3 - 2 * second;
           eb = same ? ea + 1 : 2 * second;
@@ -887,7 +897,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
         const int j = rj0 + ly, e = (j - j0) * (kTI + 1) + (k - i0);
         const int ex = k - ri0, eu = ly * kRW + (ex >> 5);
         const uint32_t ebit = 1u << (ex & 31);
-        if (slot >= CAP) {
+        if (__builtin_expect(slot >= CAP, 0)) {
           atomicOr(&M.ovf[eu], ebit);
           continue;
         }
@@ -905,12 +915,12 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
             int pe = __ffs(em & ~(1 << in)) - 1;  // partner()
             if (em == 15) pe = (q & 1) == getb(M.zb, ox, oy) ? in ^ 1 : 3 - in;
             (side ? C.p4 : C.p1) =
-                (uint16_t)(((oy + (pe == 2)) * kRX + ox + (pe == 1)) | (pe & 1 ? kKindV : 0));
+                (uint16_t)(pack_xy(ox + (pe == 1), oy + (pe == 2)) | (pe & 1 ? kKindV : 0));
             fl |= side ? CF_P4 : CF_P1;
           }
         }
         C.fl = fl;
-        C.edge = (uint16_t)e;
+        C.edge = (uint16_t)pack_xy(k - i0, j - j0);
         C.ord = (uint8_t)((ri0 + lx - (k - 2)) * 2 + second);
         {  // push the slot on the edge's list: a head of kHB bits in a shared word
           uint32_t* hw = &M.head[e / kHPW];
@@ -951,27 +961,31 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
     for (int b0 = 0; b0 < 2 * ncand; b0 += kTileThreads) {
       const int item = b0 + vt, side = item & 1;
       Cand& C = M.u.c.cand[min(item >> 1, CAP - 1)];
-      int k = 0, j = 0;
-      bool act = item < 2 * ncand;
-      if (act) {
-        k = i0 + C.edge % (kTI + 1);
-        j = j0 + C.edge / (kTI + 1);
-        act = !getb(M.ovf, k - ri0, j - rj0);  // else the edge is done in place
-      }
-      // the pair shares the chord: the even lane converts A and forms cx,
-      // the odd lane B and cy, and they swap (shuffles instead of FP64 work)
-      double px = 0.0, py = 0.0;
-      float pxf = 0.0f, pyf = 0.0f, fy_t = 0.0f;
-      if (act) {
-        if constexpr (sizeof(R) == 4) {
-          // the state reads this lane needs, issued together
-          const uint8_t fl = C.fl;
-          const float fy_ab = TV.own_fraction(side ? C.b : C.a);
-          if (fl & (side ? CF_P4 : CF_P1)) fy_t = TV.own_fraction(side ? C.p4 : C.p1);
-          TV.xyf(side ? C.b : C.a, k, j, fy_ab, &px, &py, &pxf, &pyf);
-        } else {
-          TV.xy(side ? C.b : C.a, k, j, &px, &py);
+      const int k = i0 + lx_of(C.edge), j = j0 + ly_of(C.edge);
+      // an edge that is done in place takes no fit here
+      const bool act = item < 2 * ncand && !getb(M.ovf, k - ri0, j - rj0);
+      // the pair shares the chord: the even lane forms A and cx, the odd lane
+      // B and cy, and they swap (shuffles instead of FP64 work)
+      const bool third = act && (C.fl & (side ? CF_P4 : CF_P1));
+      double px = 0.0, py = 0.0, X = 0.0, Y = 0.0, org = 0.0;
+      float pxf = 0.0f, pyf = 0.0f, Xf = 0.0f, Yf = 0.0f;
+      if constexpr (sizeof(R) == 4) {
+        const uint16_t r = side ? C.b : C.a, r3 = side ? C.p4 : C.p1;
+        // the state reads this lane needs, issued together
+        const float fy = act ? TV.own_fraction(r) : 0.0f, fy3 = third ? TV.own_fraction(r3) : 0.0f;
+        bool plain = !act || TV.xy_shifted(r, k, j, fy, &px, &py, &pxf, &pyf);
+        if (third) plain = TV.xy_shifted(r3, k, j, fy3, &X, &Y, &Xf, &Yf) && plain;
+        org = (double)kShift;
+        const unsigned odd_sums = __ballot_sync(kFull, !plain);
+        if (__builtin_expect(odd_sums != 0u, 0) && (odd_sums >> (lane & 30) & 3u)) {
+          // a pair with a sum of the other kind takes its points relative to (k, j)
+          org = 0.0;
+          xy_rare(TV, r, k, j, &px, &py);
+          if (third) xy_rare(TV, r3, k, j, &X, &Y);
         }
+      } else {
+        if (act) TV.xy(side ? C.b : C.a, k, j, &px, &py);
+        if (third) TV.xy(side ? C.p4 : C.p1, k, j, &X, &Y);
       }
       const double ox = __shfl_xor_sync(kFull, px, 1), oy = __shfl_xor_sync(kFull, py, 1);
       const float oxf = __shfl_xor_sync(kFull, pxf, 1), oyf = __shfl_xor_sync(kFull, pyf, 1);
@@ -983,44 +997,36 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       const double cx = side ? od : dd, cy = side ? dd : od;
       const double sq = dd * dd, osq = __shfl_xor_sync(kFull, sq, 1);
       const double c2 = side ? osq + sq : sq + osq;  // cx*cx + cy*cy
-      const double x0 = -ax;
-      const bool online = d_eq0(bx);
+      // A relative to (k, j): x0 = -x, y0 = y (exact)
+      double x0 = -ax, y0 = ay;
+      if constexpr (sizeof(R) == 4) {
+        const double v = (side ? ay : org) - (side ? org : ax), ov = __shfl_xor_sync(kFull, v, 1);
+        x0 = side ? ov : v;
+        y0 = side ? v : ov;
+      }
+      const bool online = d_eq0(bx) || (sizeof(R) == 4 && dbits(bx) == dbits(org));
       // the third point, then the circle.  The warp's lanes come together
       // between the two, so that those whose point takes longer do not run
       // the circle's FP64 chain a second time.
       double ys = 0.0;
       bool ok = false;
-      const bool want = act && !online && !line_only && !d_below_sep(c2) && (C.fl & (side ? CF_P4 : CF_P1));
+      const bool want = third && !online && !line_only && !d_below_sep(c2);
       const unsigned wanted = __ballot_sync(kFull, want);
       if (want) {
-        double X, Y, rx, ry, r2;
+        double rx = X - ax, ry = Y - ay, r2 = rx * rx + ry * ry;
         bool tfar, use = true;
-        if constexpr (sizeof(R) == 4) {
-          // its offsets from A exactly; its distance from B only where a float
-          // estimate (error below 2e-6 per component) does not already put it
-          // clearly past the minimum separation
-          float Xf, Yf;
-          TV.xyf(side ? C.p4 : C.p1, k, j, fy_t, &X, &Y, &Xf, &Yf);
-          rx = X - ax;
-          ry = Y - ay;
-          r2 = rx * rx + ry * ry;
-          const float txf = Xf - bxf, tyf = Yf - byf;
-          if (txf * txf + tyf * tyf >= 1.5e-4f) {
-            tfar = true;
-          } else {
-            const double tx = X - bx, ty = Y - by;
-            tfar = !d_below_sep(tx * tx + ty * ty);
-          }
+        // in the FP32 form the distance from B only where a float estimate
+        // (error below 2e-6 per component) does not already put it clearly
+        // past the minimum separation
+        const float txf = Xf - bxf, tyf = Yf - byf;
+        if (sizeof(R) == 4 && txf * txf + tyf * tyf >= 1.5e-4f) {
+          tfar = true;
         } else {
-          TV.xy(side ? C.p4 : C.p1, k, j, &X, &Y);
-          const FitPt third = fit_pt(X, Y, ax, ay, bx, by);
-          rx = third.rx;
-          ry = third.ry;
-          r2 = third.r2;
-          tfar = !d_below_sep(third.t2);
+          const double tx = X - bx, ty = Y - by;
+          tfar = !d_below_sep(tx * tx + ty * ty);
         }
-        if (side ? !tfar : d_below_sep(r2)) {  // too close to B (A): the next marker
-          const NextPt q = next_point(TV, item >> 1, side, k, j, ax, ay, bx, by);
+        if (__builtin_expect(side ? !tfar : d_below_sep(r2), 0)) {  // too close to B (A): the next marker
+          const NextPt q = next_point(TV, item >> 1, side, k, j, ax - org, ay - org, bx - org, by - org);
           use = q.found;
           rx = q.T.rx;
           ry = q.T.ry;
@@ -1028,7 +1034,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
           tfar = !d_below_sep(q.T.t2);
         }
         __syncwarp(wanted);
-        if (use) ok = circle_cross_r(ay, x0, cx, cy, c2, rx, ry, r2, tfar, &ys);
+        if (use) ok = circle_cross_r(y0, x0, cx, cy, c2, rx, ry, r2, tfar, &ys);
       }
       const double yo = __shfl_xor_sync(kFull, ys, 1);
       const bool oko = __shfl_xor_sync(kFull, (int)ok, 1) != 0;
@@ -1036,7 +1042,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
         double y;
         int kind;
         if (online) {
-          y = by;
+          y = by - org;
           kind = D_FIT_ONLINE;
         } else if (ok && oko) {
           y = d_scale<-1>(ys + yo);
@@ -1045,7 +1051,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
           y = ok ? ys : yo;
           kind = D_FIT_ONE;
         } else {  // no circle: the chord's own crossing
-          y = ay + (x0 * cy) / cx;
+          y = y0 + (x0 * cy) / cx;
           kind = D_FIT_LINE;
         }
         C.y = y;
@@ -1066,7 +1072,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
     n_inv = 0;
 #pragma unroll 1
     for (int w = tid; w < ne; w += kTileThreads) {
-      const int id = M.u.c.le[w], ex = id % kRX, ey = id / kRX;
+      const int id = M.u.c.le[w], ex = lx_of(id), ey = ly_of(id);
       if (getb(M.ovf, ex, ey)) continue;
       const int k = ri0 + ex, j = rj0 + ey;
       const int e = (j - j0) * (kTI + 1) + (k - i0);
@@ -1075,7 +1081,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
       const uint32_t hd = (M.head[e / kHPW] >> ((e % kHPW) * kHB)) & kHNone;
       int kept = -1;
       NewV<R> nv;
-      if (hd != kHNone && M.u.c.next[hd] < 0 && present) {
+      if (__builtin_expect(hd != kHNone && M.u.c.next[hd] < 0 && present, 1)) {
         // one candidate on an edge that keeps a marker: it is the marker
         kept = (int)hd;
         nv.present = 1;
@@ -1098,7 +1104,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
           return q == 5 || q == 10;
         };
         const bool fr = four(ex), fl = four(ex - 1);
-        if (fr || fl) M.vrl[e] = verdicts_of(TV, kept, k, fr, fl);
+        if (__builtin_expect(fr || fl, 0)) M.vrl[e] = verdicts_of(TV, kept, k, fr, fl);
       }
       if (own && nv.present) {
         if (AX) { if (in_range((long long)k * P + j, G.d.nH())) out.sH[(long long)k * P + j] = nv.s; }
