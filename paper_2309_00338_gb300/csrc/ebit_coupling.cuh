@@ -53,11 +53,12 @@ __device__ __forceinline__ R face_force(const Fluids<R>& f, R ka, R kb, R ca, R 
 constexpr int kCR2 = 8;  // rows per block of the column-pair kernel
 
 template <typename R, int CR = kCR2, int NB = 4>
-__global__ void __launch_bounds__(kCT) k_coupling(const R* __restrict__ C, const R* __restrict__ kap,
+__global__ void __launch_bounds__(kCT) k_coupling(const R* C, const R* kap,
                                                   Dims d, Fluids<R> f, R* __restrict__ rho,
                                                   R* __restrict__ mu, R* __restrict__ fx,
                                                   R* __restrict__ fy) {
   static_assert(CR % NB == 0, "strip of whole batches");
+  chained_start();
   using R2 = typename std::conditional<sizeof(R) == 4, float2, double2>::type;
   const int i0 = 2 * (blockIdx.x * kCT + threadIdx.x);
   const int lane = threadIdx.x & 31;
@@ -71,11 +72,11 @@ __global__ void __launch_bounds__(kCT) k_coupling(const R* __restrict__ C, const
   const bool pairs = (d.nx & 1) == 0;  // rows of nx elements keep pairs aligned
   auto load = [&](const R* p, int row, R* a, R* b) {
     if (c1) {
-      const R2 v = __ldg(reinterpret_cast<const R2*>(p + (long long)row * d.P + i0));
+      const R2 v = *reinterpret_cast<const R2*>(p + (long long)row * d.P + i0);
       *a = v.x;
       *b = v.y;
     } else if (c0) {
-      *a = __ldg(p + (long long)row * d.P + i0);
+      *a = p[(long long)row * d.P + i0];
     }
   };
   R cb0 = R(0), kb0 = nan, cb1 = R(0), kb1 = nan;  // row below, columns i0, i0 + 1
@@ -95,8 +96,8 @@ __global__ void __launch_bounds__(kCT) k_coupling(const R* __restrict__ C, const
         load(kap, j, &ka[q], &kc[q]);
       }
       if (j < jc && left) {
-        cl[q] = __ldg(&C[(long long)j * d.P + i0 - 1]);
-        kl[q] = __ldg(&kap[(long long)j * d.P + i0 - 1]);
+        cl[q] = C[(long long)j * d.P + i0 - 1];
+        kl[q] = kap[(long long)j * d.P + i0 - 1];
       }
     }
 #pragma unroll
@@ -195,12 +196,13 @@ __device__ __forceinline__ void mix_run(const MixRing& M, unsigned head, const F
 
 // Same grid, layouts and outputs as k_coupling.
 template <int CR = kCR, int NB = 2>
-__global__ void __launch_bounds__(kCT) k_coupling_q(const double* __restrict__ C,
-                                                    const double* __restrict__ kap, Dims d,
+__global__ void __launch_bounds__(kCT) k_coupling_q(const double* C,
+                                                    const double* kap, Dims d,
                                                     Fluids<double> f, double* __restrict__ rho,
                                                     double* __restrict__ mu, double* __restrict__ fx,
                                                     double* __restrict__ fy) {
   static_assert(CR % NB == 0, "strip of whole batches");
+  chained_start();
   __shared__ FaceRing face_ring[kCT / 32];
   __shared__ MixRing mix_ring[kCT / 32];
   FaceRing& F = face_ring[threadIdx.x >> 5];
@@ -218,8 +220,8 @@ __global__ void __launch_bounds__(kCT) k_coupling_q(const double* __restrict__ C
   const bool props = rho || mu;
   double cb = 0.0, kb = nan;
   if (j0 > 0 && cell) {
-    cb = __ldg(&C[(long long)(j0 - 1) * d.P + i]);
-    kb = __ldg(&kap[(long long)(j0 - 1) * d.P + i]);
+    cb = C[(long long)(j0 - 1) * d.P + i];
+    kb = kap[(long long)(j0 - 1) * d.P + i];
   }
   for (int jb = j0; jb < j1; jb += NB) {
     double c[NB], k[NB], cl[NB], kl[NB];
@@ -231,12 +233,12 @@ __global__ void __launch_bounds__(kCT) k_coupling_q(const double* __restrict__ C
       cl[q] = 0.0;
       kl[q] = nan;
       if (j < jc && cell) {
-        c[q] = __ldg(&C[(long long)j * d.P + i]);
-        k[q] = __ldg(&kap[(long long)j * d.P + i]);
+        c[q] = C[(long long)j * d.P + i];
+        k[q] = kap[(long long)j * d.P + i];
       }
       if (j < jc && left) {
-        cl[q] = __ldg(&C[(long long)j * d.P + i - 1]);
-        kl[q] = __ldg(&kap[(long long)j * d.P + i - 1]);
+        cl[q] = C[(long long)j * d.P + i - 1];
+        kl[q] = kap[(long long)j * d.P + i - 1];
       }
     }
 #pragma unroll

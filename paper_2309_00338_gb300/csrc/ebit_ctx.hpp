@@ -81,8 +81,14 @@ struct ebit_ctx {
   double* partial = nullptr;
   double* area = nullptr;
   unsigned* area_done = nullptr;    // tiles of the fields launch done (reset by its last tile)
+  // counters and largest CFL number (cfl_bits = ctr + kCounters); a step's
+  // first sweep counts into first_ctr and sets ctr to zero, its second sweep
+  // and its fields launch count into ctr, and the latter adds first_ctr to ctr
+  // and sets it to zero: no launch of the step only clears memory
   unsigned long long* ctr = nullptr;
   unsigned long long* cfl_bits = nullptr;
+  unsigned long long* first_ctr = nullptr;
+  bool first_dirty = false;         // a step ended before its fields launch
   int* status = nullptr;
   int* ghf_list = nullptr;          // EBIT_CURV_GHF: cells left without kappa
   unsigned* ghf_count = nullptr;

@@ -30,11 +30,27 @@
 
 namespace ebit {
 
+// Every kernel of the step sequence begins with chained_start(): its launch is
+// programmatic (launch_chained), so its blocks may already be resident, and it
+// touches no memory before the launches ahead of it are complete and their
+// writes visible.  What those may have written is therefore not read-only for
+// this kernel's lifetime: it is read with ordinary loads, and pointers to it
+// are neither __restrict__ nor read with __ldg, whose loads may be moved ahead
+// of the wait.
+__device__ __forceinline__ void chained_start() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next launch of the chain come onto the SMs once every block of this
+// one got here or ended.  Late in the block: allowed from the block's start,
+// the next launch's blocks crowded onto the SMs that this one left first (a
+// step of 1024^2 cells took 83 us, and 77 with the call before the last phase;
+// 91 without chaining; 64^2 cells 38, 36 and 51).
+__device__ __forceinline__ void chained_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+
 enum {
   D_NH = 0, D_NV, D_CANCELLED, D_ZSET, D_ZCONFLICT, D_FIT_ONLINE, D_FIT_LINE, D_FIT_ONE,
   D_FIT_TWO, D_WALL_CLAMP, D_INVARIANT, D_HF_INVALID, D_CFL, D_NUSED
 };
 constexpr int kCounters = 16;
+constexpr int kCounterWords = kCounters + 1;  // the counters, then the bits of the largest CFL number
 enum { ST_CFL = 1, ST_INVARIANT = 2, ST_TIMEOUT = 4 };
 
 // Two points closer than 0.01 cell do not define a usable circle (Sec. 2.2).
@@ -106,19 +122,19 @@ __device__ __forceinline__ uint32_t span_mask(int wi, int a, int b) {
   return up & ~((1u << lo) - 1u);
 }
 
-// Loads of the state a kernel advances.  LD = 0: through the read-only
-// (non-coherent) cache, for kernels that never write what they read; LD = 1:
+// Loads of the state a kernel advances.  LD = 0: ordinary (L1 and L2), for
+// kernels that never write what they read; LD = 1:
 // cached in L2 only (coherent), for a kernel that reads, after a fenced count
 // of finished tiles, what other blocks of the same launch wrote.
 template <int LD, typename T>
 __device__ __forceinline__ T ld_state(const T* p) {
   if constexpr (LD != 0) return __ldcg(p);
-  else return __ldg(p);
+  else return *p;
 }
 
 // Bits x0 .. x0+31 of a stored row of nw words (bits outside the row read 0).
 template <int LD = 0>
-__device__ __forceinline__ uint32_t row_bits(const uint32_t* __restrict__ row, int nw, int x0) {
+__device__ __forceinline__ uint32_t row_bits(const uint32_t* row, int nw, int x0) {
   const int q = x0 >> 5, r = x0 & 31;
   const uint32_t a = (q >= 0 && q < nw) ? ld_state<LD>(&row[q]) : 0u;
   const uint32_t b = (q + 1 >= 0 && q + 1 < nw) ? ld_state<LD>(&row[q + 1]) : 0u;
@@ -782,11 +798,11 @@ __device__ NewV<R> new_unaligned(const A& S, bool line_only, int k, int j, int* 
 // ---------------------------------------------------------------------------
 template <typename R, int AX, int LD = 0>
 struct GView {
-  const uint32_t* __restrict__ K;
-  const uint32_t* __restrict__ Z;
-  const R* __restrict__ sH;
-  const R* __restrict__ sV;
-  const R* __restrict__ w;  // velocity component along the sweep, (ny+1)x(nx+1)
+  const uint32_t* K;
+  const uint32_t* Z;
+  const R* sH;
+  const R* sV;
+  const R* w;  // velocity component along the sweep, (ny+1)x(nx+1)
   Dims d;
   R lam;
   __device__ __forceinline__ int tnx() const { return AX ? d.ny : d.nx; }
@@ -811,7 +827,7 @@ struct GView {
   }
   __device__ __forceinline__ R vel(int i, int j) const {
     const long long q = AX ? (long long)i * (d.nx + 1) + j : (long long)j * (d.nx + 1) + i;
-    return in_range(q, d.nW()) ? __ldg(&w[q]) : R(0);
+    return in_range(q, d.nW()) ? w[q] : R(0);
   }
   __device__ __forceinline__ int corners(int i, int j) const {
     return k(i, j) | (k(i + 1, j) << 1) | (k(i + 1, j + 1) << 2) | (k(i, j + 1) << 3);

@@ -37,13 +37,13 @@ template <typename R> __host__ __device__ constexpr int fields_min_blocks() { re
 // a and b), each the marker's fraction or its one-minus: one sequence for all
 // of them, so that a warp whose cells differ repeats no FP64 work.
 template <typename R>
-__device__ __forceinline__ double fraction_of(int q, int zc, const R* __restrict__ sH, const R* __restrict__ sV,
+__device__ __forceinline__ double fraction_of(int q, int zc, const R* sH, const R* sV,
                                               const Dims& d, int i, int j) {
   const long long q0 = (long long)j * d.P + i;
   // exact conversions on the integer pipe
   auto marker = [&](int e) {
     const long long at = e == 1 ? q0 + 1 : e == 2 ? q0 + d.P : q0;
-    return in_range(at, e & 1 ? d.nV() : d.nH()) ? to_d<R>(__ldg(e & 1 ? &sV[at] : &sH[at])) : 0.0;
+    return in_range(at, e & 1 ? d.nV() : d.nH()) ? to_d<R>(e & 1 ? sV[at] : sH[at]) : 0.0;
   };
   const int em = edge_mask(q);
   if (em != 15) {
@@ -197,6 +197,9 @@ struct AreaSum {
   long long n = 0;
   double scale = 0.0;
   double* area = nullptr;
+  // the counters of the step's first sweep, which block (0, 0) adds to the
+  // launch's own and sets to zero
+  unsigned long long* first = nullptr;
 };
 
 // The tile (bx, by) of one grid; its area partial goes to partial[slot].
@@ -204,9 +207,9 @@ struct AreaSum {
 // appended to it (ghf_count, zeroed before the launch, counts them): one
 // global atomic per tile reserves its slice.
 template <typename R>
-__device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
-                                            const uint32_t* __restrict__ Z,
-                                            const R* __restrict__ sH, const R* __restrict__ sV,
+__device__ __forceinline__ void fields_tile(const uint32_t* K,
+                                            const uint32_t* Z,
+                                            const R* sH, const R* sV,
                                             const Dims& d, R dx, R* C, R* kappa, double* partial,
                                             long long slot, unsigned long long* ctr, int bx, int by,
                                             int* ghf_list = nullptr, unsigned* ghf_count = nullptr,
@@ -375,6 +378,7 @@ __device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
     }
   }
 
+  chained_next();
   // height-function curvature of the tile's interface cells
   for (int e = tid; e < nlist; e += kFieldThreads) {
     const int ci = lst[e], ly = ci / kFP, lx = ci - ly * kFP - 1;
@@ -385,10 +389,10 @@ __device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
     int seg[2][2];
     const int ns = segments(q, edge_mask(q) == 15 ? fgetb(zw, lx, ly) : 0, seg);
     const long long q0 = (long long)j * d.P + i, q2 = q0 + d.P;
-    const R px[4] = {in_range(q0, d.nH()) ? __ldg(&sH[q0]) : R(0), R(1),
-                     in_range(q2, d.nH()) ? __ldg(&sH[q2]) : R(0), R(0)};
-    const R py[4] = {R(0), in_range(q0 + 1, d.nV()) ? __ldg(&sV[q0 + 1]) : R(0), R(1),
-                     in_range(q0, d.nV()) ? __ldg(&sV[q0]) : R(0)};
+    const R px[4] = {in_range(q0, d.nH()) ? sH[q0] : R(0), R(1),
+                     in_range(q2, d.nH()) ? sH[q2] : R(0), R(0)};
+    const R py[4] = {R(0), in_range(q0 + 1, d.nV()) ? sV[q0 + 1] : R(0), R(1),
+                     in_range(q0, d.nV()) ? sV[q0] : R(0)};
     const bool ycol = heights_along_y(ns, seg, px, py);
     bool valid = ycol ? (i - 1 >= 0 && i + 1 <= d.nx - 1 && j - 3 >= 0 && j + 3 <= d.ny - 1)
                       : (j - 1 >= 0 && j + 1 <= d.ny - 1 && i - 3 >= 0 && i + 3 <= d.nx - 1);
@@ -476,10 +480,17 @@ __device__ __forceinline__ void fields_tile(const uint32_t* __restrict__ K,
 
 template <typename R>
 __global__ void __launch_bounds__(field_threads<R>(), fields_min_blocks<R>())
-k_fields_tile(const uint32_t* __restrict__ K, const uint32_t* __restrict__ Z,
-              const R* __restrict__ sH, const R* __restrict__ sV, Dims d, R dx, R* C, R* kappa,
+k_fields_tile(const uint32_t* K, const uint32_t* Z,
+              const R* sH, const R* sV, Dims d, R dx, R* C, R* kappa,
               double* partial, unsigned long long* ctr, int* ghf_list, unsigned* ghf_count,
               AreaSum sum) {
+  chained_start();
+  if (sum.first && blockIdx.x + blockIdx.y == 0 && threadIdx.x < kCounterWords) {
+    const unsigned long long v = sum.first[threadIdx.x];
+    sum.first[threadIdx.x] = 0ull;
+    if (v && threadIdx.x < kCounters) atomicAdd(&ctr[threadIdx.x], v);
+    if (v && threadIdx.x == kCounters) atomicMax(&ctr[kCounters], v);  // bits of a positive double
+  }
   fields_tile<R>(K, Z, sH, sV, d, dx, C, kappa, partial,
                  (long long)blockIdx.y * gridDim.x + blockIdx.x, ctr, blockIdx.x, blockIdx.y, ghf_list,
                  ghf_count, sum);
@@ -510,6 +521,7 @@ struct FieldItem {
 template <typename R>
 __global__ void __launch_bounds__(field_threads<R>(), fields_min_blocks<R>())
 k_fields_tile_batch(const FieldDesc<R>* __restrict__ descs, const FieldItem* __restrict__ items) {
+  chained_start();
   const FieldItem it = items[blockIdx.x];
   const FieldDesc<R>& D = descs[it.grid];
   fields_tile<R>(D.K, D.Z, D.sH, D.sV, D.d, D.dx, D.C, D.kappa, D.partial,

@@ -28,9 +28,9 @@ static_assert(D_NUSED <= D_HF_OTHER && D_HF_MARKERS < kCounters, "counter slots"
 
 constexpr int kGhfThreads = 128;  // k_ghf_fit block
 
-__device__ __forceinline__ int kbit(const uint32_t* __restrict__ K, int kw, int i, int j, long long n) {
+__device__ __forceinline__ int kbit(const uint32_t* K, int kw, int i, int j, long long n) {
   const long long q = (long long)j * kw + (i >> 5);
-  return in_range(q, n) ? (__ldg(&K[q]) >> (i & 31)) & 1 : 0;
+  return in_range(q, n) ? (K[q] >> (i & 31)) & 1 : 0;
 }
 
 // Read-only view of the state and fractions of one context.
@@ -46,15 +46,15 @@ struct GhfView {
   __device__ int z(int i, int j) const { return kbit(Z, d.zw, i, j, d.nZ()); }
   __device__ R c(int i, int j) const {
     const long long q = (long long)j * d.P + i;
-    return in_range(q, d.nV()) ? __ldg(&C[q]) : R(0);
+    return in_range(q, d.nV()) ? C[q] : R(0);
   }
   __device__ R h(int i, int j) const {
     const long long q = (long long)j * d.P + i;
-    return in_range(q, d.nH()) ? __ldg(&sH[q]) : R(0);
+    return in_range(q, d.nH()) ? sH[q] : R(0);
   }
   __device__ R v(int i, int j) const {
     const long long q = (long long)j * d.P + i;
-    return in_range(q, d.nV()) ? __ldg(&sV[q]) : R(0);
+    return in_range(q, d.nV()) ? sV[q] : R(0);
   }
 };
 
@@ -153,15 +153,16 @@ struct ParabolaFit {
 
 template <typename R>
 __global__ void __launch_bounds__(kGhfThreads, 6)
-    k_ghf_fit(GhfView<R> S, R dx, const int* __restrict__ list, const unsigned* __restrict__ count,
-              R* __restrict__ kappa, unsigned long long* __restrict__ ctr) {
+    k_ghf_fit(GhfView<R> S, R dx, const int* list, const unsigned* count, R* kappa,
+              unsigned long long* ctr) {
+  chained_start();
   __shared__ unsigned s_cnt[3];
   if (threadIdx.x < 3) s_cnt[threadIdx.x] = 0;
   __syncthreads();
   const unsigned n = *count;
   unsigned got[3] = {0, 0, 0};
   for (unsigned e = blockIdx.x * kGhfThreads + threadIdx.x; e < n; e += gridDim.x * kGhfThreads) {
-    const int idx = __ldg(&list[e]);
+    const int idx = list[e];
     const int i = idx % S.d.nx, j = idx / S.d.nx;
     const int c[4] = {S.k(i, j), S.k(i + 1, j), S.k(i + 1, j + 1), S.k(i, j + 1)};
     const int q = c[0] | (c[1] << 1) | (c[2] << 2) | (c[3] << 3);

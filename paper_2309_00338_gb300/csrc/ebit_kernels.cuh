@@ -295,8 +295,9 @@ __global__ void k_store_frac(const R* __restrict__ src, int w, int h, long long 
 // 16-byte words and the destination is 16-byte aligned (the pitched rows
 // always are), else the element type itself.
 template <typename W>
-__global__ void k_unpitch(const W* __restrict__ src, long long pitch, W* __restrict__ dst, long long w,
+__global__ void k_unpitch(const W* src, long long pitch, W* __restrict__ dst, long long w,
                           int h) {
+  chained_start();
   const long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= w) return;
   for (long long y = blockIdx.y; y < h; y += gridDim.y) dst[y * w + x] = src[y * pitch + x];

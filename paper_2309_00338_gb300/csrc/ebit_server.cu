@@ -47,6 +47,7 @@
 #include "ebit_ctx.hpp"
 #include "ebit_fields.cuh"
 #include "ebit_ghf.cuh"
+#include "ebit_launch.hpp"
 #include "ebit_persist.cuh"
 #include "ebit_tile.cuh"
 
@@ -103,11 +104,13 @@ struct AreaDesc {
 // the batched fields launch lists into them.
 template <typename R>
 __global__ void k_ghf_reset(const ebit::FieldDesc<R>* __restrict__ descs, int n) {
+  ebit::chained_start();
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g < n && descs[g].ghf_count) *descs[g].ghf_count = 0u;
 }
 
 __global__ void k_area_batch(const AreaDesc* __restrict__ descs) {
+  ebit::chained_start();
   const AreaDesc D = descs[blockIdx.x];
   __shared__ double red[256];
   double acc = 0.0;
@@ -124,6 +127,7 @@ __global__ void k_area_batch(const AreaDesc* __restrict__ descs) {
 // Every grid's status word, gathered into host-mapped memory at the end of a
 // batch step (one thread per grid).
 __global__ void k_status_gather(int* const* __restrict__ status, int n, int* out) {
+  ebit::chained_start();
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g < n) out[g] = *status[g];
 }
@@ -407,12 +411,13 @@ struct Group {
       const ebit::PersistCtl P{d_ctl, d_need, n_items0, (int)n, budget_ns};
       ebit::k_sweep_persistent<R><<<persist_blocks, ebit::tile_threads<R>(), smem, st>>>(d_s0, d_s1, d_items0, P);
     } else {
-      ebit::k_sweep_tile_both<R, ebit::batch_cand_cap<R>()><<<n_items0, ebit::tile_threads<R>(), smem, st>>>(d_s0, d_s1, d_items0);
-      ebit::k_sweep_tile_both<R, ebit::batch_cand_cap<R>()><<<n_items0, ebit::tile_threads<R>(), smem, st>>>(d_s0 + n, d_s1 + n, d_items0);
+      const auto sweep = ebit::k_sweep_tile_both<R, ebit::batch_cand_cap<R>()>;
+      ebit_detail::launch_chained(sweep, n_items0, ebit::tile_threads<R>(), smem, st, d_s0, d_s1, d_items0);
+      ebit_detail::launch_chained(sweep, n_items0, ebit::tile_threads<R>(), smem, st, d_s0 + n, d_s1 + n, d_items0);
     }
     if (!ghf.empty()) k_ghf_reset<R><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(d_fd, (int)n);
-    ebit::k_fields_tile_batch<R><<<n_fitems, ebit::field_threads<R>(), 0, st>>>(d_fd, d_fitems);
-    k_area_batch<<<(unsigned)n, 256, 0, st>>>(d_ad);
+    ebit_detail::launch_chained(ebit::k_fields_tile_batch<R>, n_fitems, ebit::field_threads<R>(), 0, st, d_fd, d_fitems);
+    ebit_detail::launch_chained(k_area_batch, (unsigned)n, 256, 0, st, d_ad);
     for (const int g : ghf) {  // the state is back in the buffer the plan was built on
       const ebit_ctx* c = inst[g]->ctx;
       const int b = c->cur;
@@ -722,7 +727,7 @@ ebit_status ebit_server::launch_all() {
   if (a != EBIT_OK) return a;
   if ((a = g64.launch(stream, persistent, budget_ns)) != EBIT_OK) return a;
   const size_t n = stepping.size();
-  k_status_gather<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(d_status, (int)n, h_status_dev);
+  ebit_detail::launch_chained(k_status_gather, (unsigned)((n + 127) / 128), 128, 0, stream, d_status, (int)n, h_status_dev);
   return cudaGetLastError() == cudaSuccess ? EBIT_OK : fail_s(EBIT_ECUDA, "status gather launch");
 }
 

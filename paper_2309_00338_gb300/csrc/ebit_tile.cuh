@@ -1165,6 +1165,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
     __syncthreads();
   }
 
+  chained_next();
   // P7: colour words.  Lane L of warp ow (0 or 1) takes tile row j0 + L and
   // the 32 vertices / cells i0 + 32 ow + b; the y sweep transposes them into
   // stored rows.  Centre colours of new four-marker cells (all four edges
@@ -1230,11 +1231,14 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
   }
 }
 
-// One grid: block (bx, by) runs the tile at (64 bx, 32 by).
+// One grid: block (bx, by) runs the tile at (64 bx, 32 by).  zero: a set of
+// counters no tile of this launch adds to, set to zero for the next ones.
 template <typename R, int AX, int T>
 __global__ void __launch_bounds__(T, T == tile_threads<R>() ? tile_min_blocks<R>() : 4)
 k_sweep_tile(GView<R, AX> G, Buf<R> out, int line_only, unsigned long long* ctr,
-             unsigned long long* cfl_bits, int* status) {
+             unsigned long long* cfl_bits, int* status, unsigned long long* zero) {
+  chained_start();
+  if (zero && blockIdx.x + blockIdx.y == 0 && threadIdx.x < kCounterWords) zero[threadIdx.x] = 0ull;
   sweep_tile<R, AX, 0, kCandCap, T>(G, out, line_only, ctr, cfl_bits, status, blockIdx.x * kTI, blockIdx.y * kTJ);
 }
 
@@ -1256,15 +1260,6 @@ struct WorkItem {
   int grid, tx, ty;
 };
 
-template <typename R, int AX>
-__global__ void __launch_bounds__(tile_threads<R>(), tile_min_blocks<R>())
-k_sweep_tile_batch(const SweepDesc<R, AX>* __restrict__ descs, const WorkItem* __restrict__ items) {
-  const WorkItem it = items[blockIdx.x];
-  const SweepDesc<R, AX>& D = descs[it.grid];
-  if (!D.active) return;
-  sweep_tile<R, AX>(D.G, D.out, D.line_only, D.ctr, D.cfl_bits, D.status, it.tx * kTI, it.ty * kTJ);
-}
-
 // Square grids only: a grid's tiles are the same in both sweep directions, so
 // one launch can take the first (or second) sweep of every grid, each tile in
 // the direction its grid's split order puts there (x first on even steps):
@@ -1273,6 +1268,7 @@ template <typename R, int CAP = kCandCap>
 __global__ void __launch_bounds__(tile_threads<R>(), tile_min_blocks<R>())
 k_sweep_tile_both(const SweepDesc<R, 0>* __restrict__ dx, const SweepDesc<R, 1>* __restrict__ dy,
                   const WorkItem* __restrict__ items) {
+  chained_start();
   const WorkItem it = items[blockIdx.x];
   const SweepDesc<R, 0>& X = dx[it.grid];
   if (X.active) {

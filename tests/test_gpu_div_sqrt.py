@@ -48,7 +48,9 @@ def _values(rng, n, span):
     m = np.where(kind == 2, m % np.uint64(4), np.where(kind == 3, np.uint64((1 << 52) - 1) - m % np.uint64(4), m))
     e = (1023 + rng.integers(-span, span + 1, n)).astype(np.uint64)
     x = (m | (e << np.uint64(52)) | (rng.integers(0, 2, n).astype(np.uint64) << np.uint64(63))).view(np.float64)
-    sq = (x * x).view(np.uint64) + rng.integers(0, 3, n).astype(np.uint64) - np.uint64(1)
+    with np.errstate(over="ignore"):
+        square = x * x
+    sq = square.view(np.uint64) + rng.integers(0, 3, n).astype(np.uint64) - np.uint64(1)
     return np.where((kind == 4) & (span < 500), sq.view(np.float64), x)
 
 
