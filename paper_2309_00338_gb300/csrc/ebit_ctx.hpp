@@ -97,7 +97,7 @@ struct ebit_ctx {
   // next fields launch waits for
   cudaEvent_t ev_queued = nullptr, ev_c_read = nullptr;
   bool c_read_pending = false;
-  std::vector<void*> allocs;
+  void* memory = nullptr;  // the one allocation that holds the arrays above
   // per-kernel event timing (off unless ebit_set_timing)
   bool timing = false;
   struct Mark {

@@ -536,11 +536,13 @@ ebit_status ebit_server::admit(Instance* in) {
   ebit_status s = ebit_init(&in->ctx, &g, &sc, admit_stream);
   if (s != EBIT_OK) return s;
   const size_t esz = r.prec == EBIT_FP32 ? 4 : 8;
-  const size_t vb = (size_t)(r.n + 1) * (r.n + 1) * esz;
-  if (cudaMalloc(&in->u, vb) != cudaSuccess || cudaMalloc(&in->v, vb) != cudaSuccess) {
+  const size_t vb = ((size_t)(r.n + 1) * (r.n + 1) * esz + 255) / 256 * 256;
+  if (cudaMalloc(&in->u, 2 * vb) != cudaSuccess) {
     cudaGetLastError();
+    in->u = nullptr;
     return fail_s(EBIT_ENOMEM, "velocity allocation");
   }
+  in->v = (char*)in->u + vb;  // one allocation for both
   const int nb = (int)(((long long)(r.n + 1) * (r.n + 1) + 255) / 256);
   if (r.prec == EBIT_FP32)
     k_velocity<float><<<nb, 256, 0, admit_stream>>>(r.field, r.n, 1.0 / r.n, r.omega, r.cx, r.cy, r.drift_u, r.drift_v, (float*)in->u, (float*)in->v);
@@ -589,7 +591,6 @@ void ebit_server::retire(size_t idx) {
   }
   ebit_destroy(in->ctx);
   cudaFree(in->u);
-  cudaFree(in->v);
   {
     std::lock_guard<std::mutex> lk(mu);
     done[in->ticket] = res;
@@ -834,7 +835,6 @@ void ebit_server::admit_all(std::vector<std::unique_ptr<Instance>>& admitted) {
       r.status = s;
       if (in->ctx) ebit_destroy(in->ctx);
       if (in->u) cudaFree(in->u);
-      if (in->v) cudaFree(in->v);
       std::lock_guard<std::mutex> lk(mu);
       done[in->ticket] = r;
       pending.erase(in->ticket);
