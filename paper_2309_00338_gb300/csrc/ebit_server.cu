@@ -320,7 +320,7 @@ struct Group {
         (cudaGetDevice(&dev) != cudaSuccess ||
          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ebit::k_sweep_persistent<R>,
-                                                       ebit::tile_threads<R>(),
+                                                       ebit::batch_threads<R>(),
                                                        ebit::tile_smem_bytes<R, ebit::batch_cand_cap<R>()>()) != cudaSuccess)) {
       cudaGetLastError();
       per_sm = -1;
@@ -409,11 +409,11 @@ struct Group {
       cudaMemcpyAsync(d_need, h_need, n * sizeof(unsigned), cudaMemcpyHostToDevice, st);
       cudaMemsetAsync(d_ctl, 0, (n + 1) * sizeof(unsigned), st);
       const ebit::PersistCtl P{d_ctl, d_need, n_items0, (int)n, budget_ns};
-      ebit::k_sweep_persistent<R><<<persist_blocks, ebit::tile_threads<R>(), smem, st>>>(d_s0, d_s1, d_items0, P);
+      ebit::k_sweep_persistent<R><<<persist_blocks, ebit::batch_threads<R>(), smem, st>>>(d_s0, d_s1, d_items0, P);
     } else {
       const auto sweep = ebit::k_sweep_tile_both<R, ebit::batch_cand_cap<R>()>;
-      ebit_detail::launch_chained(sweep, n_items0, ebit::tile_threads<R>(), smem, st, d_s0, d_s1, d_items0);
-      ebit_detail::launch_chained(sweep, n_items0, ebit::tile_threads<R>(), smem, st, d_s0 + n, d_s1 + n, d_items0);
+      ebit_detail::launch_chained(sweep, n_items0, ebit::batch_threads<R>(), smem, st, d_s0, d_s1, d_items0);
+      ebit_detail::launch_chained(sweep, n_items0, ebit::batch_threads<R>(), smem, st, d_s0 + n, d_s1 + n, d_items0);
     }
     if (!ghf.empty()) k_ghf_reset<R><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(d_fd, (int)n);
     ebit_detail::launch_chained(ebit::k_fields_tile_batch<R>, n_fitems, ebit::field_threads<R>(), 0, st, d_fd, d_fitems);

@@ -69,10 +69,19 @@ template <typename R> __host__ __device__ constexpr int tile_threads() { return 
 template <typename R> __host__ __device__ constexpr int tile_min_blocks();
 template <> __host__ __device__ constexpr int tile_min_blocks<float>() { return 7; }
 template <> __host__ __device__ constexpr int tile_min_blocks<double>() { return 6; }
-constexpr int kMkCap = 1536;  // markers of a region held in shared memory
+// Markers of a region held in shared memory: as many as fit in the carve-outs
+// that seven (six) tiles take anyway; 2048 cost 5% of the sweep (less L1).
+template <typename R> __host__ __device__ constexpr int marker_cap() { return sizeof(R) == 4 ? 1792 : 1632; }
+// Block shape of the batched kernels, whose code of both directions makes more
+// warps share what each fetches: 256 uneven grids in one batch advance 2.12e10
+// (FP32) and 1.69e10 (FP64) cells a second with six warps a tile, 2.02 and
+// 1.64 with four, 2.10 and 1.70 with five, 2.03 and 1.66 with seven (four and
+// three tiles per SM).
+template <typename R> __host__ __device__ constexpr int batch_threads() { return 192; }
+template <typename R> __host__ __device__ constexpr int batch_min_blocks() { return sizeof(R) == 4 ? 5 : 4; }
 // Candidates per tile of the batched kernels: many small grids of uneven
 // sizes hold more interface per tile than one large grid, and the longer
-// list (16-bit heads) still leaves 4 (FP32) / 3 (FP64) tiles per SM.
+// list (16-bit heads) still leaves 5 (FP32) / 4 (FP64) tiles per SM.
 template <typename R> __host__ __device__ constexpr int batch_cand_cap() {
   return sizeof(R) == 4 ? 511 : 383;
 }
@@ -98,7 +107,7 @@ struct Cand {
 template <typename R, int CAP = kCandCap>
 struct TileMem {
   static_assert(CAP <= 65534, "candidate slots fit the 16-bit heads");
-  static constexpr int kCap = CAP;
+  static constexpr int kCap = CAP, kMkCap = marker_cap<R>();
   union {
     uint16_t mk[kMkCap];       // P1-P3: region index of every marker, by rank
     struct {
@@ -619,7 +628,7 @@ __device__ __forceinline__ void sweep_tile(const GView<R, AX, LD>& G, const Buf<
   __shared__ unsigned long long s_dmax;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kTileThreads = T;
+  constexpr int kTileThreads = T, kMkCap = marker_cap<R>();
   constexpr int kWarps = kTileThreads / 32;
   const int tnx = G.tnx(), tny = G.tny();
   const int ri0 = i0 - 4, rj0 = j0 - 2;
@@ -1265,18 +1274,18 @@ struct WorkItem {
 // the direction its grid's split order puts there (x first on even steps):
 // the x descriptor when it is active for this launch, else the y one.
 template <typename R, int CAP = kCandCap>
-__global__ void __launch_bounds__(tile_threads<R>(), tile_min_blocks<R>())
+__global__ void __launch_bounds__(batch_threads<R>(), batch_min_blocks<R>())
 k_sweep_tile_both(const SweepDesc<R, 0>* __restrict__ dx, const SweepDesc<R, 1>* __restrict__ dy,
                   const WorkItem* __restrict__ items) {
   chained_start();
   const WorkItem it = items[blockIdx.x];
   const SweepDesc<R, 0>& X = dx[it.grid];
   if (X.active) {
-    sweep_tile<R, 0, 0, CAP>(X.G, X.out, X.line_only, X.ctr, X.cfl_bits, X.status, it.tx * kTI,
+    sweep_tile<R, 0, 0, CAP, batch_threads<R>()>(X.G, X.out, X.line_only, X.ctr, X.cfl_bits, X.status, it.tx * kTI,
                              it.ty * kTJ);
   } else {
     const SweepDesc<R, 1>& Y = dy[it.grid];
-    sweep_tile<R, 1, 0, CAP>(Y.G, Y.out, Y.line_only, Y.ctr, Y.cfl_bits, Y.status, it.tx * kTI,
+    sweep_tile<R, 1, 0, CAP, batch_threads<R>()>(Y.G, Y.out, Y.line_only, Y.ctr, Y.cfl_bits, Y.status, it.tx * kTI,
                              it.ty * kTJ);
   }
 }
