@@ -328,6 +328,10 @@ ebit_status init_scene(ebit_ctx* c, const ebit_scene* scene) {
       cudaStreamSynchronize(c->stream);
     } else {
       cudaMemsetAsync(unused, 0, A.bytes(), c->stream);
+      // nothing waits for the copies here, and where the GPU reads pageable
+      // memory itself they may still be running: the context keeps their
+      // sources until it is destroyed
+      for (auto* v : {&circ, &curve, &notch}) c->scene_host.push_back(std::move(*v));
     }
   };
   ebit_status s;

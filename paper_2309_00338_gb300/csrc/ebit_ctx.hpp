@@ -98,6 +98,7 @@ struct ebit_ctx {
   cudaEvent_t ev_queued = nullptr, ev_c_read = nullptr;
   bool c_read_pending = false;
   void* memory = nullptr;  // the one allocation that holds the arrays above
+  std::vector<std::vector<double>> scene_host;  // sources of the scene's copies to the device
   // per-kernel event timing (off unless ebit_set_timing)
   bool timing = false;
   struct Mark {
