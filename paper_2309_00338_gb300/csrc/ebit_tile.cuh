@@ -520,7 +520,7 @@ __device__ __noinline__ NewV<R> new_unaligned_rare(const A S, bool line_only, in
 
 // The tile with origin (i0, j0) by the generic logic, every answer recomputed
 // from global memory: for the tiles whose region holds more markers than
-// shared memory keeps (over a quarter of its edges, as noise does), so that
+// shared memory keeps (about a third of its edges, as noise does), so that
 // any state is swept.
 template <typename R, int AX, int LD, int T>
 __device__ __noinline__ void tile_in_place(const GView<R, AX, LD> G, const Buf<R> out, int line_only,
