@@ -133,8 +133,12 @@ __device__ __forceinline__ float height_kappa(const float h[3], float dx) {
   return -hpp / den;
 }
 __device__ __forceinline__ double height_kappa(const fix60 h[3], double dx) {
-  const double hp = d_scale<-1>(from_fix60((long long)(h[2] - h[0])));
-  const double hpp = from_fix60((long long)((h[2] - h[1]) - (h[1] - h[0])));
+  // With one end cell full and the other empty a height lies in [1, 6] cells:
+  // first differences are below 5 cells, which a signed word of 2^-60 cells
+  // holds (8), and the second difference is below 10, which takes units of 2^-59.
+  const long long up = (long long)(h[2] - h[1]), down = (long long)(h[1] - h[0]);
+  const double hp = d_scale<-1>(from_fix60(up + down));
+  const double hpp = d_scale<1>(from_fix60((up >> 1) - (down >> 1)));
   const double qv = 1.0 + hp * hp;
   const double den = dx * (qv * d_sqrt(qv));
   return -d_div(hpp, den);
