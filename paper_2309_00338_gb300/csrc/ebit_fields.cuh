@@ -9,8 +9,8 @@
 // exactly: C and a NaN kappa are stored four cells at a time from the words,
 // and the interface cells, listed in region order, overwrite theirs.  FP64
 // work is confined to them, and there to what has to be double: the area is
-// added up as integers (exactly, in any order) and so are the heights of the
-// double form.  What bounds it then is instruction issue and the dense stores:
+// added up as integers (in any order; a tile with next to no area in double)
+// and so are the heights of the double form.  What bounds it then is instruction issue and the dense stores:
 // 4096^2 cells with 1.2 M interface cells, 118 -> 88 us in FP32 and 322 -> 140
 // us in FP64 (with double heights and sums the FP64 pipe was busy 82% of the
 // time); 2.2 and 2.9 TB/s of the dense model, state read and C, kappa written.
@@ -101,6 +101,25 @@ __device__ __forceinline__ double from_fix60(long long v) {
   const unsigned long long sig = p > 52 ? a >> (p - 52) : a << (52 - p);
   return __longlong_as_double((long long)((v < 0 ? 1ull << 63 : 0ull) |
                                           ((unsigned long long)(1023 + p - 60) << 52) | (sig & (kImplicit - 1))));
+}
+
+// The area of a tile's listed interface cells (of the region; those of its halo
+// are left out) in double, by one warp in a fixed order: every lane gets the sum.
+// Units of 2^-60 lose relative accuracy on areas far below a cell; few tiles
+// hold nothing else, so this is out of line.
+template <typename R>
+__device__ __noinline__ double small_area(const uint16_t* lst, int n, const uint32_t* kw, const uint32_t* zw,
+                                          const R* sH, const R* sV, const Dims d, int rx0, int ry0) {
+  double a = 0.0;
+#pragma unroll 1
+  for (int e = threadIdx.x & 31; e < n; e += 32) {
+    const int t = lst[e] & 0x7fff, ly = t / kFP, lx = t - ly * kFP - 1;
+    if (lx < kFH || lx >= kFH + kFX || ly < kFH || ly >= kFH + kFY) continue;
+    a = a + fraction_of(fcorners(kw, lx, ly), fgetb(zw, lx, ly), sH, sV, d, rx0 + lx, ry0 + ly);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a = a + __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
 }
 
 // What the height functions add up.  The float form adds floats in stencil
@@ -228,7 +247,10 @@ __device__ __forceinline__ void fields_tile(const uint32_t* K,
   __shared__ __align__(16) HT cs[kFRY * kFP];  // fractions of the region
   __shared__ uint16_t lst[kFRY * kFRX];        // interface cells, in region order (entries of cs)
   __shared__ int s_cnt[D_NUSED];
-  __shared__ unsigned long long s_area;  // the tile's area, units of 2^-52 cells
+  // the tile's area: full cells, and its interface cells' in units of 2^-60
+  // cells, s_area + s_area_hi 2^48
+  __shared__ unsigned long long s_area;
+  __shared__ unsigned s_area_hi, s_full;
   __shared__ unsigned s_nghf, s_ghf_base;
   __shared__ int s_last, s_n;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -237,6 +259,7 @@ __device__ __forceinline__ void fields_tile(const uint32_t* K,
   if (tid < D_NUSED) s_cnt[tid] = 0;
   if (tid == 0) {
     s_area = 0ull;
+    s_area_hi = s_full = 0u;
     s_nghf = 0u;
   }
   // region columns / rows inside the grid
@@ -287,7 +310,7 @@ __device__ __forceinline__ void fields_tile(const uint32_t* K,
   }
   {
     const int fsum = __reduce_add_sync(0xffffffffu, full);
-    if (lane == 0 && fsum) atomicAdd(&s_area, (unsigned long long)fsum << 52);
+    if (lane == 0 && fsum) atomicAdd(&s_full, (unsigned)fsum);
   }
   __syncthreads();
 
@@ -347,7 +370,7 @@ __device__ __forceinline__ void fields_tile(const uint32_t* K,
   __syncthreads();
 
   // interface fractions (FP64 on full warps) and the tile's area, added up as
-  // integers: exactly, whatever the order
+  // integers: the same in any order
   const int nlist = s_n;
   fix60 acc = 0;  // at most 11 cells a thread: below 2^64
   static_assert((kFRY * kFRX + kFieldThreads - 1) / kFieldThreads <= 15, "a thread's area fits");
@@ -363,22 +386,35 @@ __device__ __forceinline__ void fields_tile(const uint32_t* K,
     }
   }
   if (__any_sync(0xffffffffu, acc != 0)) {
-    const unsigned long long a = (acc + 128) >> 8;  // units of 2^-52, below 2^56
-    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)a & 0xffffffu);
-    const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(a >> 24) & 0xffffffu);
-    const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(a >> 48));
-    if (lane == 0) atomicAdd(&s_area, lo + ((unsigned long long)mid << 24) + ((unsigned long long)hi << 48));
+    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)acc & 0xffffffu);
+    const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(acc >> 24) & 0xffffffu);
+    const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(acc >> 48));
+    if (lane == 0) {
+      atomicAdd(&s_area, lo + ((unsigned long long)mid << 24));
+      atomicAdd(&s_area_hi, hi);
+    }
   }
   __syncthreads();
   // the tile's partial, and its count towards the launch's last tile, by the
-  // last thread: it rarely has curvature work, so the fence and the counter's
+  // last warp: it rarely has curvature work, so the fence and the counter's
   // round trip overlap the other threads' curvature
-  if (tid == kFieldThreads - 1) {
-    partial[slot] = __ull2double_rn(s_area) * 0x1p-52;
-    s_last = 0;
-    if (sum.done) {
-      __threadfence();  // the partial is visible before the count says so
-      s_last = atomicAdd(sum.done, 1u) == (unsigned)(sum.n - 1);
+  if (warp == kFieldThreads / 32 - 1) {
+    const unsigned hi = s_area_hi, full = s_full;
+    const unsigned long long lo = s_area, units = lo + ((unsigned long long)(hi & 0xffffu) << 48);
+    double p = (__ull2double_rn(lo) * 0x1p-60 + (double)hi * 0x1p-12) + (double)full;
+    // Each cell's area is cut by less than a unit, and only below 2^-8.  Where
+    // the cells hold fewer than 2^50 units on average (that many keep the
+    // relative error below 2^-50) and no full cell outweighs them, they are
+    // added in double.
+    if (full == 0u && hi < 0x10000u && units != 0u && units < (unsigned long long)nlist << 50)
+      p = small_area<R>(lst, nlist, kw, zw, sH, sV, d, rx0, ry0);
+    if (lane == 31) {
+      partial[slot] = p;
+      s_last = 0;
+      if (sum.done) {
+        __threadfence();  // the partial is visible before the count says so
+        s_last = atomicAdd(sum.done, 1u) == (unsigned)(sum.n - 1);
+      }
     }
   }
 
