@@ -260,13 +260,15 @@ __device__ __forceinline__ uint32_t upto32(int c0, int last) {
 }
 
 
-// n + f + kShift for a grid line number n and a fraction f (see xy_shifted).
+// n + f + kShift for a grid line number n and a fraction f (see xy_shifted);
+// false unless f is +0 or in [2^-26, 1) (-0, whose sign bit counts as part of
+// the exponent here, is not).
 constexpr int kShift = 12;
 __device__ __forceinline__ bool shifted_sum(int n, float f, double* s) {
   const unsigned u = __float_as_uint(f), e = u >> 23;
   const unsigned long long m = (unsigned long long)(u ? (u & 0x7fffffu) | 0x800000u : 0u) << ((e - 101u) & 31u);
   *s = __longlong_as_double((1026ll << 52) + ((long long)(n + kShift - 8) << 49) + (long long)m);
-  return (unsigned)(n + 4) < 8u && (u == 0u || e >= 101u);
+  return (unsigned)(n + 4) < 8u && (u == 0u || e - 101u < 26u);
 }
 
 // Accessor of the tile for the shared sweep logic (beyond, walk,
