@@ -151,7 +151,7 @@ ebit_status launch_fields(ebit_ctx* c) {
                              (const R*)c->C, L.d};
     const long long cells = (long long)L.d.nx * L.d.ny;
     const int blocks = (int)std::min<long long>((cells + ebit::kGhfThreads - 1) / ebit::kGhfThreads,
-                                                152LL * 8);
+                                                8LL * c->sms);
     // an ordinary launch: its work sits in its first blocks, and these have to
     // spread over all SMs, not over those that the fields launch leaves first
     // (2048^2 cells: the step with its coupling takes 201 us, 225 chained)
@@ -208,7 +208,7 @@ ebit_status launch_sweep(ebit_ctx* c, const void* vel, double lam, unsigned long
     // (a sweep of 1024^2 cells, 561 tiles: 33.1 us against 35.4 in FP32; 1021
     // x 771 in FP64 20.2 against 22.1; eight warps 39.5 and 20.6)
     constexpr int kWide = 192;
-    const bool wide = (long long)grid.x * grid.y <= 4 * 152;
+    const bool wide = (long long)grid.x * grid.y <= 4 * c->sms;
     static bool attr = false;  // once per instantiation and process
     if (!attr) {
       EBIT_CK(cudaFuncSetAttribute(ebit::k_sweep_tile<R, AX, ebit::tile_threads<R>()>,
@@ -261,7 +261,10 @@ ebit_status new_ctx(ebit_ctx** out, const ebit_grid* grid, void* stream) {
   c->grid = *grid;
   c->L = layout_of(grid);
   c->stream = (cudaStream_t)stream;
-  const ebit_status s = alloc_ctx(c);
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
+  const ebit_status s = e == cudaSuccess ? alloc_ctx(c) : fail(EBIT_ECUDA, "device: %s", cudaGetErrorString(e));
   if (s != EBIT_OK) {
     free_ctx(c);
     delete c;

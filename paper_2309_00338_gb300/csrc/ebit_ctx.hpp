@@ -71,6 +71,7 @@ struct ebit_ctx {
   ebit_grid grid;
   ebit_detail::Layout L;
   cudaStream_t stream = nullptr;
+  int sms = 0;  // of the context's device
   uint32_t* K[2] = {nullptr, nullptr};
   uint32_t* Z[2] = {nullptr, nullptr};
   void* sH[2] = {nullptr, nullptr};

@@ -423,7 +423,7 @@ struct Group {
       const int b = c->cur;
       const ebit::GhfView<R> S{c->K[b], c->Z[b], (const R*)c->sH[b], (const R*)c->sV[b], (const R*)c->C, c->L.d};
       const long long cells = (long long)c->L.d.nx * c->L.d.ny;
-      const int blocks = (int)std::min<long long>((cells + ebit::kGhfThreads - 1) / ebit::kGhfThreads, 152LL * 8);
+      const int blocks = (int)std::min<long long>((cells + ebit::kGhfThreads - 1) / ebit::kGhfThreads, 8LL * c->sms);
       ebit::k_ghf_fit<R><<<blocks, ebit::kGhfThreads, 0, st>>>(S, (R)c->grid.dx, c->ghf_list, c->ghf_count,
                                                               (R*)c->kappa, c->ctr);
     }
