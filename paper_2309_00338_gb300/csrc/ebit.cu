@@ -261,10 +261,11 @@ ebit_status new_ctx(ebit_ctx** out, const ebit_grid* grid, void* stream) {
   c->grid = *grid;
   c->L = layout_of(grid);
   c->stream = (cudaStream_t)stream;
+  ebit_status s = alloc_ctx(c);
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
-  const ebit_status s = e == cudaSuccess ? alloc_ctx(c) : fail(EBIT_ECUDA, "device: %s", cudaGetErrorString(e));
+  if (s == EBIT_OK && (cudaGetDevice(&dev) != cudaSuccess ||
+                       cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess))
+    s = fail(EBIT_ECUDA, "device query: %s", cudaGetErrorString(cudaGetLastError()));
   if (s != EBIT_OK) {
     free_ctx(c);
     delete c;
