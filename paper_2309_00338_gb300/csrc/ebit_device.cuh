@@ -30,8 +30,9 @@
 
 namespace ebit {
 
-// Every kernel of the step sequence begins with chained_start(): its launch is
-// programmatic (launch_chained), so its blocks may already be resident, and it
+// Every kernel of the step sequence begins with chained_start(): where its launch
+// is programmatic (launch_chained; all but those of the generalised fallbacks,
+// k_ghf_fit and k_ghf_reset, are), its blocks may already be resident, and it
 // touches no memory before the launches ahead of it are complete and their
 // writes visible.  What those may have written is therefore not read-only for
 // this kernel's lifetime: it is read with ordinary loads, and pointers to it
@@ -434,8 +435,12 @@ template <> __device__ __forceinline__ double to_d<double>(double x) { return x;
 // pipes, for the circle fits: long division and longhand square root with
 // quotient digits guessed from a float reciprocal (Knuth, The Art of Computer
 // Programming 2, 4.3.1), the remainder kept exactly modulo 2^64.  Two digits
-// leave at most 2^10 units of the last place, so the remainder fits 63 bits;
-// the third digit is exact to half a unit, and the remainder's size against
+// leave at most 412 units of the last place for the quotient and 274 for the
+// root (the first digit's error, below 2^-21, times the reciprocal's, below
+// 2^-23, and the roundings; taken over every 24-bit leading part of the divisor
+// or radicand and every approximation within its stated error).  The remainder
+// is at most that many times 2^53, and 2^54: below 0.41 and 0.54 of 2^63.  The
+// third digit is exact to half a unit, and the remainder's size against
 // the divisor rounds it.  The results are the IEEE ones, bit for bit.  About
 // 50 integer instructions each, a dozen cycles of an SM's four issue slots,
 // against 16 cycles for every FP64 instruction that they replace: the sweep of

@@ -10,10 +10,11 @@
 // and the interface cells, listed in region order, overwrite theirs.  FP64
 // work is confined to them, and there to what has to be double: the area is
 // added up as integers (in any order; a tile with next to no area in double)
-// and so are the heights of the double form.  What bounds it then is instruction issue and the dense stores:
-// 4096^2 cells with 1.2 M interface cells, 118 -> 88 us in FP32 and 322 -> 140
-// us in FP64 (with double heights and sums the FP64 pipe was busy 82% of the
-// time); 2.2 and 2.9 TB/s of the dense model, state read and C, kappa written.
+// and so are the heights of the double form.  What bounds it then is instruction
+// issue and the dense stores: 4096^2 cells with 1.2 M interface cells, 118 -> 91
+// us in FP32 and 322 -> 142 us in FP64 (with double heights and sums the FP64 pipe
+// was busy 82% of the time); 3.0 and 3.8 TB/s of the dense model, state read and
+// C, kappa written.
 #pragma once
 #include "ebit_device.cuh"
 
@@ -26,8 +27,8 @@ constexpr int kFW = 3;                                     // words per region b
 constexpr int kFP = 72;  // row pitch of the region's fractions: cell lx is entry lx + 1, so that
                          // groups of four entries are groups of four of the tile's columns
 // Threads per tile and blocks per SM the kernel is compiled for: 4096^2 cells
-// take 88 us in FP32 with eight blocks of 32 registers (a few spilled), 99 with
-// six, 111 with five; in FP64 140 us with six, 143 with five, 171 with seven.
+// take 91 us in FP32 with eight blocks of 32 registers (a few spilled), 98 with
+// six, 109 with five; in FP64 142 us with six and with five, 171 with seven.
 template <typename R> __host__ __device__ constexpr int field_threads() { return 256; }
 template <typename R> __host__ __device__ constexpr int fields_min_blocks() { return sizeof(R) == 4 ? 8 : 6; }
 
