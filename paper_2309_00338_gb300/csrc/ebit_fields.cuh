@@ -94,23 +94,24 @@ __device__ __forceinline__ fix60 to_fix60(double f) {
   if (sh <= 0) return sig << -sh;
   return sh > 52 ? 1ull : sig >> sh;
 }
-// (double)v 2^-60 for |v| < 2^63, to 53 bits (rounded toward zero).
-__device__ __forceinline__ double from_fix60(long long v) {
+// (double)v 2^-U for |v| < 2^63, to 53 bits (rounded toward zero).
+template <int U>
+__device__ __forceinline__ double from_fix(long long v) {
   if (v == 0) return 0.0;
   const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
   const int p = 63 - __clzll((long long)a);
   const unsigned long long sig = p > 52 ? a >> (p - 52) : a << (52 - p);
   return __longlong_as_double((long long)((v < 0 ? 1ull << 63 : 0ull) |
-                                          ((unsigned long long)(1023 + p - 60) << 52) | (sig & (kImplicit - 1))));
+                                          ((unsigned long long)(1023 + p - U) << 52) | (sig & (kImplicit - 1))));
 }
 
 // The area of a tile's listed interface cells (of the region; those of its halo
 // are left out) in double, by one warp in a fixed order: every lane gets the sum.
 // Units of 2^-60 lose relative accuracy on areas far below a cell; few tiles
-// hold nothing else, so this is out of line.
+// hold nothing else.
 template <typename R>
-__device__ __noinline__ double small_area(const uint16_t* lst, int n, const uint32_t* kw, const uint32_t* zw,
-                                          const R* sH, const R* sV, const Dims d, int rx0, int ry0) {
+__device__ __forceinline__ double small_area(const uint16_t* lst, int n, const uint32_t* kw, const uint32_t* zw,
+                                             const R* sH, const R* sV, const Dims& d, int rx0, int ry0) {
   double a = 0.0;
 #pragma unroll 1
   for (int e = threadIdx.x & 31; e < n; e += 32) {
@@ -121,6 +122,15 @@ __device__ __noinline__ double small_area(const uint16_t* lst, int n, const uint
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) a = a + __shfl_xor_sync(0xffffffffu, a, o);
   return a;
+}
+
+// a 2^-12 + b 2^-60 for a < 2^24 and b < 2^48, rounded, on the integer pipe.
+__device__ __forceinline__ double tile_area(unsigned a, unsigned long long b) {
+  if (a == 0u) return from_fix<60>((long long)b);
+  const int p = 31 - __clz((int)a), drop = p - 4;  // bits of b beyond the 53
+  unsigned long long sig = ((unsigned long long)a << (52 - p)) + (drop >= 0 ? b >> drop : b << -drop);
+  if (drop > 0) sig += (b >> (drop - 1)) & 1u;
+  return __longlong_as_double((long long)(((unsigned long long)(1023 - 12 + p) << 52) + (sig - kImplicit)));
 }
 
 // What the height functions add up.  The float form adds floats in stencil
@@ -157,8 +167,8 @@ __device__ __forceinline__ double height_kappa(const fix60 h[3], double dx) {
   // first differences are below 5 cells, which a signed word of 2^-60 cells
   // holds (8), and the second difference is below 10, which takes units of 2^-59.
   const long long up = (long long)(h[2] - h[1]), down = (long long)(h[1] - h[0]);
-  const double hp = d_scale<-1>(from_fix60(up + down));
-  const double hpp = d_scale<1>(from_fix60((up >> 1) - (down >> 1)));
+  const double hp = from_fix<61>(up + down);  // half their sum
+  const double hpp = from_fix<59>((up >> 1) - (down >> 1));
   const double qv = 1.0 + hp * hp;
   const double den = dx * (qv * d_sqrt(qv));
   return -d_div(hpp, den);
@@ -400,14 +410,14 @@ __device__ __forceinline__ void fields_tile(const uint32_t* K,
   // last warp: it rarely has curvature work, so the fence and the counter's
   // round trip overlap the other threads' curvature
   if (warp == kFieldThreads / 32 - 1) {
-    const unsigned hi = s_area_hi, full = s_full;
-    const unsigned long long lo = s_area, units = lo + ((unsigned long long)(hi & 0xffffu) << 48);
-    double p = (__ull2double_rn(lo) * 0x1p-60 + (double)hi * 0x1p-12) + (double)full;
+    const unsigned long long lo = s_area, b = lo & ((1ull << 48) - 1);
+    const unsigned a = (s_full << 12) + s_area_hi + (unsigned)(lo >> 48);  // at most 2048 cells
+    double p = tile_area(a, b);
     // Each cell's area is cut by less than a unit, and only below 2^-8.  Where
     // the cells hold fewer than 2^50 units on average (that many keep the
-    // relative error below 2^-50) and no full cell outweighs them, they are
-    // added in double.
-    if (full == 0u && hi < 0x10000u && units != 0u && units < (unsigned long long)nlist << 50)
+    // relative error below 2^-50) and there is no full cell, they are added in
+    // double.
+    if (s_full == 0u && a < 0x4000u && (a | b) != 0u && (((unsigned long long)a << 48) | b) < (unsigned long long)nlist << 50)
       p = small_area<R>(lst, nlist, kw, zw, sH, sV, d, rx0, ry0);
     if (lane == 31) {
       partial[slot] = p;
